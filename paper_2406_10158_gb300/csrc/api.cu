@@ -142,8 +142,7 @@ void free_db(gcc_db* db) {
     cudaFree(db->sort.v0);
     cudaFree(db->sort.k1);
     cudaFree(db->sort.v1);
-    cudaFree(db->sort.hist);
-    cudaFree(db->sort.totals);
+    cudaFree(db->sort.work);
     cudaFree(db->scan_tmp);
     cudaFree(db->need);
     cudaFree(db->order_key);
@@ -238,16 +237,17 @@ gcc_status create_impl(const gcc_db_desc* desc, gcc_db** out) {
     if ((s = dev_alloc(&db->sort.v0, items * 4, "sort values"))) return bail(s);
     if ((s = dev_alloc(&db->sort.k1, items * 4, "sort keys"))) return bail(s);
     if ((s = dev_alloc(&db->sort.v1, items * 4, "sort values"))) return bail(s);
-    if ((s = dev_alloc(&db->sort.hist, gcc::sort_max_tiles(items) * 256 * 4, "sort histogram")))
+    if ((s = dev_alloc(&db->sort.work, gcc::sort_work_words(items) * 4, "sort histograms")))
         return bail(s);
-    if ((s = dev_alloc(&db->sort.totals, 256 * 4, "sort totals"))) return bail(s);
+    db->sort.err = &db->st->error;
     if ((s = dev_alloc(&db->scan_tmp, gcc::scan_tmp_words(items) * 4, "scan scratch"))) return bail(s);
     if ((s = dev_alloc(&db->need, d.max_batch_ops * 4, "wait thresholds"))) return bail(s);
     if ((s = dev_alloc(&db->order_key, d.max_batch_txns * 8, "commit keys"))) return bail(s);
     if ((s = dev_alloc(&db->fold_flags, d.max_batch_txns * 8, "validity flags and ranks")))
         return bail(s);
     if (d.schema == GCC_SCHEMA_KV &&
-        (s = dev_alloc(&db->fold_seg, gcc::fold_seg_bytes(d.max_batch_ops), "fold carries")))
+        (s = dev_alloc(&db->fold_seg, gcc::fold_seg_bytes(d.max_batch_ops, d.max_batch_txns),
+                       "fold descriptors")))
         return bail(s);
     // MVCC version pointers, one per slot, zero between batches
     if (d.schema == GCC_SCHEMA_KV &&
@@ -382,9 +382,14 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
     a.queue_width = p.queue_width;
     a.queue_after = queue_after_for(p, scheme);
 
-    GCC_CK(gcc::launch_batch_begin(db->st, db->dbs, scheme, st));
-    launches += 1;
     const bool kv = db->d.schema == GCC_SCHEMA_KV;
+    // deterministic key-value batches: every record chain by prefix sums (the
+    // pipeline begins the batch itself)
+    const bool fold = scheme == GCC_DET && kv && !p.det_dataflow;
+    if (!fold) {
+        GCC_CK(gcc::launch_batch_begin(db->st, db->dbs, scheme, st));
+        launches += 1;
+    }
     if (!kv && n_ops) {
         // payments by last name become payments of the customer they name,
         // before any scheme sees the batch
@@ -393,14 +398,9 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
         a.ops = db->ops_resolved;
         launches += 1;
     }
-    // deterministic key-value batches: every record chain by prefix sums
-    const bool fold = scheme == GCC_DET && kv && !p.det_dataflow;
     if (fold) {
         GCC_CK(cudaEventRecord(rec.ev[1], st));
-        GCC_CK(gcc::det_fold_kv(a, db->d.field_bytes, db->sort, db->scan_tmp, db->fold_flags,
-                                db->fold_seg, st));
-        const int bits = bit_length((uint64_t)db->d.n_fields * db->d.n_records);
-        launches += 2 + 3 * ((bits + 7) / 8) + 4 + 1 + 3 + 2;
+        GCC_CK(gcc::det_fold_kv(a, db->d.field_bytes, db->sort, db->fold_seg, launches, st));
         GCC_CK(cudaEventRecord(rec.ev[2], st));
         GCC_CK(cudaEventRecord(rec.ev[3], st));
         rec.stream = st;
@@ -443,7 +443,7 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
         const int bits = std::max(1, bit_length(db->n_meta));
         GCC_CK(gcc::det_prepare(a, db->sort, db->scan_tmp, bits, db->d.schema, st,
                                 p.det_dataflow == 2));
-        launches += 1 + 3 * ((bits + 7) / 8) + 1 + 3 + 1;   // emit, sort, flags, scan, need
+        launches += 1 + gcc::radix_sort_launches(bits) + 1 + 3 + 1;   // emit, sort, flags, scan, need
     }
     // OCC group commit on key-value batches: units of up to gu transactions
     // (each unit's ops are staged together: at most 255 per unit)
@@ -490,7 +490,7 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
     }
     if (n_txns && (scheme == GCC_OCC || scheme == GCC_TO || scheme == GCC_MVCC)) {
         GCC_CK(gcc::densify_commit_order(a, db->sort, st));
-        launches += 1 + 3 * 4 + 1;                           // emit, 4 sort passes, rank
+        launches += 1 + gcc::radix_sort_launches(32) + 1;    // emit, sort, rank
     }
     if (n_txns && scheme == GCC_DET) {
         GCC_CK(gcc::densify_in_id_order(a, db->fold_flags, db->scan_tmp, st));
@@ -498,7 +498,7 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
     }
     if (n_txns && scheme == GCC_TICTOC) {
         GCC_CK(gcc::densify_tictoc(a, db->sort, st));
-        launches += 3 * (1 + 3 * 4) + 1;                     // 3 x (emit, 4 passes), rank
+        launches += 3 * (1 + gcc::radix_sort_launches(32)) + 1;   // 3 x (emit, sort), rank
     }
     GCC_CK(cudaEventRecord(rec.ev[3], st));
     rec.stream = st;

@@ -1,0 +1,199 @@
+// det_common.cuh -- what the deterministic scheme's passes share for key-value
+// (det_fold.cu) and order-entry (det_oe.cu) batches: the kernel that starts a
+// batch, the segmented look-back between tiles and the kernel that finishes
+// it.
+#pragma once
+
+#include <algorithm>
+
+#include "engine.cuh"
+
+namespace gcc {
+namespace {
+
+// Words of SortScratch::work between the pass tickets and the histograms.
+// The first two are left at zero by the kernel that uses them.
+enum { DW_BEGIN_DONE = 8, DW_UNTILED_ACC, DW_UNTILED, DW_VALID_DONE, DW_FINISH_TICKET };
+
+constexpr uint32_t DET_SPIN_MAX = 1u << 21;
+
+inline unsigned blocks_for(uint64_t n, int b) { return (unsigned)((n + b - 1) / b); }
+
+// A block-wide election: true in every thread of the last block to arrive at
+// `counter` (which is left at zero), whose accesses then follow every other
+// block's.
+__device__ __forceinline__ bool last_block(uint32_t* counter) {
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        fence_acq_rel();
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
+        if (last) *counter = 0;
+        fence_acq_rel();
+    }
+    __syncthreads();
+    return last;
+}
+
+// Starts a batch: zeroes the batch state, the sort's tickets, histograms and
+// first descriptor area (`zero`, `n_zero` 16-byte words, all of SortScratch::work
+// but the words above) and the pass's own descriptors (`zero2`), and checks that
+// the transactions' op ranges tile ops[0, n_ops) in id order, which the
+// contract asks for.  Where they do not, DW_UNTILED is set and the last block
+// gives every op the key `none(i)`, so that an op outside every range stays out
+// of the access table; the validation pass then overwrites the others'.
+template <class None>
+__global__ void __launch_bounds__(256)
+det_begin(const __grid_constant__ ExecArgs a, uint32_t* work, ulonglong2* zero, size_t n_zero,
+          ulonglong2* zero2, size_t n_zero2, uint32_t* keys, None none) {
+    after_previous();
+    const size_t i0 = (size_t)blockIdx.x * 256 + threadIdx.x, stride = (size_t)gridDim.x * 256;
+    if (i0 == 0) {
+        BatchState z{};
+        z.ticket_base = a.dbs->occ_clock;
+        *a.st = z;
+        for (int w = 0; w < (int)SORT_HIST; ++w)
+            if (w != DW_BEGIN_DONE && w != DW_UNTILED_ACC && w != DW_UNTILED) work[w] = 0;
+    }
+    const ulonglong2 z2 = make_ulonglong2(0ull, 0ull);
+    for (size_t i = i0; i < n_zero; i += stride) zero[i] = z2;
+    for (size_t i = i0; i < n_zero2; i += stride) zero2[i] = z2;
+    bool untiled = false;
+    for (size_t t = i0; t < a.n_txns; t += stride) {
+        const gcc_txn x = a.txns[t];
+        uint64_t before = 0;
+        if (t) {
+            const gcc_txn y = a.txns[t - 1];
+            before = (uint64_t)y.first_op + y.n_ops;
+        }
+        if (x.first_op != before) untiled = true;
+        if (t + 1 == a.n_txns && (uint64_t)x.first_op + x.n_ops != a.n_ops) untiled = true;
+    }
+    if (__syncthreads_or(untiled) && threadIdx.x == 0) atomicOr(work + DW_UNTILED_ACC, 1u);
+    if (!last_block(work + DW_BEGIN_DONE)) return;
+    const uint32_t bad = *(volatile uint32_t*)(work + DW_UNTILED_ACC);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        work[DW_UNTILED] = bad;
+        work[DW_UNTILED_ACC] = 0;
+    }
+    if (bad)
+        for (uint64_t i = threadIdx.x; i < a.n_ops; i += 256) keys[i] = none(i);
+}
+
+// The block's digit histograms: HIST_COPIES copies side by side, a lane adding
+// to the copy of its own number, so that lanes of a warp with the same digit
+// (the top digits of neighbouring ops often are) rarely meet on one word.
+constexpr int HIST_COPIES = 4;
+typedef uint32_t DigitHist[256 * HIST_COPIES];
+__device__ __forceinline__ void count_digits(DigitHist* h, uint32_t k, int bits, int passes, int digit_bits) {
+    const uint32_t copy = threadIdx.x % HIST_COPIES;
+#pragma unroll
+    for (int p = 0; p < SORT_MAX_PASSES; ++p)
+        if (p < passes) {
+            const int left = bits - p * digit_bits;
+            const uint32_t mask = (1u << (left < digit_bits ? left : digit_bits)) - 1u;
+            atomicAdd(&h[p][((k >> (p * digit_bits)) & mask) * HIST_COPIES + copy], 1u);
+        }
+}
+__device__ __forceinline__ void clear_digits(DigitHist* h) {
+#pragma unroll
+    for (int p = 0; p < SORT_MAX_PASSES; ++p)
+        for (int c = threadIdx.x; c < 256 * HIST_COPIES; c += 256) h[p][c] = 0;
+}
+
+// The block's histograms into the batch's.  Where the op ranges did not tile
+// the ops (DW_UNTILED) the counts would miss the ops outside every range: the
+// last block counts all keys instead.  Every block of the grid calls it.
+__device__ __forceinline__ void flush_digits(DigitHist* h, uint32_t* work, const uint32_t* keys,
+                                             uint64_t n, int bits, int passes, int digit_bits) {
+    const bool untiled = work[DW_UNTILED] != 0;
+    __syncthreads();
+    if (untiled) {
+        if (!last_block(work + DW_VALID_DONE)) return;
+        clear_digits(h);
+        __syncthreads();
+        for (uint64_t i = threadIdx.x; i < n; i += 256)
+            count_digits(h, *(volatile const uint32_t*)(keys + i), bits, passes, digit_bits);
+        __syncthreads();
+    }
+    for (int p = 0; p < passes; ++p) {
+        uint32_t c = 0;
+#pragma unroll
+        for (int i = 0; i < HIST_COPIES; ++i) c += h[p][threadIdx.x * HIST_COPIES + i];
+        if (c) atomicAdd(work + SORT_HIST + p * 256 + threadIdx.x, c);
+    }
+}
+
+// Ends a batch: counts the commits.  The validation pass gave every valid
+// transaction its id as its commit order, which is right when every
+// transaction is valid; otherwise the order is the rank among the valid ones,
+// by one scan over tiles of transactions with look-back (rank_desc: one zeroed
+// word per tile of 1024).
+constexpr uint32_t RANK_TILE = 1024;
+__global__ void __launch_bounds__(1024)
+det_finish(const __grid_constant__ ExecArgs a, uint32_t* work, unsigned long long* rank_desc) {
+    __shared__ uint32_t s_tile, s_warp[32], s_before;
+    constexpr unsigned long long OWN = 1ull << 62, UP_TO = 2ull << 62, MASK = (1ull << 62) - 1;
+    after_previous();
+    const unsigned long long invalid = *(volatile unsigned long long*)&a.st->invalid;
+    if (invalid == 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            a.st->committed = a.n_txns;
+            a.st->max_attempts = a.n_txns ? 1ull : 0ull;
+        }
+        return;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.st->committed = a.n_txns - invalid;
+        a.st->max_attempts = a.n_txns > invalid ? 1ull : 0ull;
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_tile = atomicAdd(work + DW_FINISH_TICKET, 1u);
+        __syncthreads();
+        const uint32_t tile = s_tile;
+        const uint64_t t = (uint64_t)tile * RANK_TILE + threadIdx.x;
+        if ((uint64_t)tile * RANK_TILE >= a.n_txns) return;
+        const bool ok = t < a.n_txns && a.results[t].status == GCC_TXN_COMMITTED;
+        const unsigned m = __ballot_sync(0xffffffffu, ok);
+        if (lane == 0) s_warp[warp] = __popc(m);
+        __syncthreads();
+        if (warp == 0) {
+            uint32_t x = s_warp[lane], inc = x;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += y;
+            }
+            s_warp[lane] = inc - x;
+            if (lane == 31) {
+                unsigned long long* d = rank_desc;
+                st_relaxed((uint64_t*)(d + tile), (tile ? OWN : UP_TO) | inc);
+                unsigned long long before = 0;
+                uint32_t spins = 0;
+                for (int64_t p = (int64_t)tile - 1; p >= 0;) {
+                    const unsigned long long w = ld_relaxed((const uint64_t*)(d + p));
+                    if (w == 0) {
+                        if (++spins > DET_SPIN_MAX) {
+                            atomicOr(&a.st->error, GCC_DEVERR_WAIT_BUDGET);
+                            break;
+                        }
+                        continue;
+                    }
+                    before += w & MASK;
+                    if (w >= UP_TO) break;
+                    --p;
+                }
+                if (tile) st_relaxed((uint64_t*)(d + tile), UP_TO | (before + inc));
+                s_before = (uint32_t)before;
+            }
+        }
+        __syncthreads();
+        if (ok) a.results[t].commit_order = s_before + s_warp[warp] + __popc(m & lanemask_lt());
+    }
+}
+
+}  // namespace
+}  // namespace gcc

@@ -11,213 +11,221 @@
 // chain with one segmented prefix sum instead of handing the record from op
 // to op, which removes the chain latency that dominates under contention.
 //
-//   validate   one warp per transaction: the same checks as the execute
-//              kernel (kinds, keys, fields, distinct keys); invalid
-//              transactions are excluded and reported INVALID
-//   emit       access table (slot = field * n_records + key, op index)
-//   sort       stable radix sort by slot: (slot, transaction id) order
-//   deltas     per sorted position the op's delta (0 for READ)
-//   scan       segmented exclusive prefix sum of the deltas, tile by tile
-//   apply      read value = initial slot value + prefix
-//   finals     last access of each slot writes initial + inclusive sum
-//   ranks      commit order = rank among valid transactions (= id when all
-//              are valid)
-#include <algorithm>
-
-#include "engine.cuh"
+//   begin      batch state, descriptors and histograms zeroed
+//   validate   a lane group per transaction: the same checks as the execute
+//              kernel (kinds, keys, fields, distinct keys); every op's access
+//              key, and the digit histograms of the sort
+//   sort       stable radix sort by (chunk, slot), slot = field * n_records +
+//              key: within a chunk, (slot, transaction id) order
+//   fold       per chunk, one kernel: segmented prefix sum of the deltas with
+//              look-back between tiles, read values out, final values in
+//   finish     commit counts; commit order where a transaction was invalid
+//
+// Chunks.  Serial execution in id order can be cut anywhere: the ops are folded
+// in chunks of consecutive positions, each starting from the table the one
+// before left.  A chunk's operands are gathered and its read values scattered
+// at random (sorted order against op order); cutting keeps the two within L2
+// (2^CHUNK_LOG2 ops: 32 MB each), where a batch of 2^24 ops at once would go
+// to DRAM sector by sector.  (Table accesses pay for it: a chunk touches the
+// table more sparsely.  On 2^24 ops over 2.5 GiB, chunks of 2^20 to 2^22 are
+// within 3 % and one chunk for all 5 % slower.)  The chunk number sorts in the
+// key's spare high bits, so the whole batch still takes one sort.
+#include "det_common.cuh"
 
 namespace gcc {
 namespace {
 
-constexpr int FB_THREADS = 1024;
-constexpr int FB_ITEMS = 4;
-constexpr int FB_TILE = FB_THREADS * FB_ITEMS;
+constexpr int FT_THREADS = 256;
+// Accesses per thread of fold_tiles.  16-byte slots hold twice the registers;
+// 2 per thread keep 4 blocks on an SM (2^24 ops: 1.52 ms for the batch against
+// 1.59 ms with 4), 8-byte slots run 4 (64 databases: 8.1 against 8.3 ms).
+template <int FB> constexpr int FT_ITEMS = FB == 16 ? 2 : 4;
+template <int FB> constexpr int FT_TILE = FT_THREADS * FT_ITEMS<FB>;
+constexpr int FT_WARPS = FT_THREADS / 32;
+constexpr int CHUNK_LOG2 = 21;
+// One sort handles at most 2^30 ops (30-bit digit counts, 31-bit positions);
+// longer batches are sorted and folded in that many at a time.
+constexpr int SORT_LOG2 = 30;
 
 __device__ __forceinline__ uint32_t d_key(uint64_t d) { return (uint32_t)d; }
 __device__ __forceinline__ uint32_t d_field(uint64_t d) { return (uint32_t)(d >> 32) & 0xffu; }
 __device__ __forceinline__ uint32_t d_kind(uint64_t d) { return (uint32_t)(d >> 40) & 0xffu; }
 
+// The sort keys of a batch: bits 0..slot_bits-1 the slot (n_slots: none),
+// above it the op's chunk, bit 31 (when free) whether the op is an ADD.
+struct FoldKeys {
+    uint32_t n_slots;
+    int slot_bits, bits, passes, digit_bits, chunk_log2;
+    int flagged;
+    __host__ __device__ uint32_t chunk_of(uint64_t op) const {
+        return (uint32_t)(op & ((1ull << SORT_LOG2) - 1)) >> chunk_log2;
+    }
+    __device__ uint32_t key(uint64_t op, uint32_t slot, bool add) const {
+        uint32_t k = slot | (bits > slot_bits ? chunk_of(op) << slot_bits : 0u);
+        return k | (flagged && add ? 0x80000000u : 0u);
+    }
+    __device__ uint32_t slot(uint32_t k) const {
+        return slot_bits == 32 ? k : k & ((1u << slot_bits) - 1u);
+    }
+    // the op of a sorted value, positions counting from op0
+    __device__ uint64_t op(uint64_t op0, uint32_t v) const { return op0 + (flagged ? v & 0x7fffffffu : v); }
+    __device__ uint32_t operator()(uint64_t op) const { return key(op, n_slots, false); }
+};
+
+FoldKeys fold_keys(uint64_t n_slots, uint64_t n_ops) {
+    FoldKeys f;
+    f.n_slots = (uint32_t)n_slots;
+    f.slot_bits = 0;
+    for (uint64_t v = n_slots; v; v >>= 1) ++f.slot_bits;
+    const uint64_t m = std::min<uint64_t>(n_ops, 1ull << SORT_LOG2);
+    int want = 0;                            // chunk bits
+    while (((uint64_t)1 << (CHUNK_LOG2 + want)) < m) ++want;
+    f.flagged = f.slot_bits <= 31;
+    const int room = f.flagged ? 31 - f.slot_bits : 0;
+    const int chunk_bits = std::min(want, room);
+    f.chunk_log2 = CHUNK_LOG2 + (want - chunk_bits);
+    f.bits = f.slot_bits + chunk_bits;
+    const SortPlan sp = sort_plan(f.bits);
+    f.passes = sp.passes;
+    f.digit_bits = sp.digit_bits;
+    return f;
+}
+
 // A running sum in the slot's lane arithmetic.
 struct Sum {
-    uint64_t lo, hi;       // hi kept modulo 2^16
+    uint64_t lo;
+    uint32_t hi;           // modulo 2^16
 };
-__device__ __forceinline__ Sum sum_add(Sum a, Sum b) {
-    return Sum{a.lo + b.lo, (a.hi + b.hi) & 0xFFFFull};
-}
-// Segmented-scan element: `head` marks the first access of a slot.
-struct Seg {
-    uint32_t head;
-    Sum v;
+__device__ __forceinline__ Sum sum_add(Sum a, Sum b) { return Sum{a.lo + b.lo, (a.hi + b.hi) & 0xFFFFu}; }
+
+// Scratch (zeroed by det_begin): one ticket per chunk, one word per tile of
+// transactions (det_finish), one descriptor per tile of ops.
+struct FoldScratch {
+    uint32_t* tickets;
+    unsigned long long* rank_desc;
+    ulonglong2* tile_desc;
+    ulonglong2* zero;
+    size_t n_zero;
 };
-// Scratch of the fold: the tile carries, then one cached delta per op.
-size_t fold_carry_bytes(size_t n_ops) {
-    return (((n_ops + FB_TILE - 1) / FB_TILE + 1) * sizeof(Seg) + 255) & ~size_t(255);
-}
-// a followed by b
-__device__ __forceinline__ Seg seg_combine(Seg a, Seg b) {
-    return Seg{a.head | b.head, b.head ? b.v : sum_add(a.v, b.v)};
-}
-
-__device__ __forceinline__ Seg shfl_up_seg(Seg s, int o) {
-    Seg r;
-    r.head = __shfl_up_sync(0xffffffffu, s.head, o);
-    r.v.lo = __shfl_up_sync(0xffffffffu, s.v.lo, o);
-    r.v.hi = __shfl_up_sync(0xffffffffu, s.v.hi, o);
-    return r;
-}
-
-// Block-wide exclusive segmented scan of one element per thread; also
-// returns the block's inclusive total.
-__device__ Seg block_seg_exclusive(Seg x, Seg* warp_tot, Seg* total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nw = blockDim.x >> 5;
-    Seg inc = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const Seg up = shfl_up_seg(inc, o);
-        if (lane >= o) inc = seg_combine(up, inc);
-    }
-    Seg exc = shfl_up_seg(inc, 1);
-    if (lane == 0) exc = Seg{0u, Sum{0, 0}};
-    if (lane == 31) warp_tot[warp] = inc;
-    __syncthreads();
-    if (warp == 0) {
-        Seg w = lane < nw ? warp_tot[lane] : Seg{0u, Sum{0, 0}};
-        Seg wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const Seg up = shfl_up_seg(wi, o);
-            if (lane >= o) wi = seg_combine(up, wi);
-        }
-        Seg we = shfl_up_seg(wi, 1);
-        if (lane == 0) we = Seg{0u, Sum{0, 0}};
-        if (lane < nw) warp_tot[lane] = we;
-        if (lane == nw - 1) warp_tot[32] = wi;
-    }
-    __syncthreads();
-    const Seg r = seg_combine(warp_tot[warp], exc);
-    if (total) *total = warp_tot[32];
-    __syncthreads();
-    return r;
+size_t rounded(size_t bytes) { return (bytes + 255) & ~size_t(255); }
+size_t chunks_of(uint64_t n_ops) { return (size_t)(n_ops >> CHUNK_LOG2) + 2; }
+FoldScratch fold_scratch(void* base, uint64_t n_ops, uint64_t n_txns) {
+    char* p = static_cast<char*>(base);
+    FoldScratch s;
+    s.zero = reinterpret_cast<ulonglong2*>(p);
+    s.tickets = reinterpret_cast<uint32_t*>(p);
+    p += rounded(chunks_of(n_ops) * 4);
+    s.rank_desc = reinterpret_cast<unsigned long long*>(p);
+    p += rounded((n_txns / RANK_TILE + 1) * 8);
+    s.tile_desc = reinterpret_cast<ulonglong2*>(p);
+    p += rounded((n_ops / FT_TILE<16> + 2) * 16);
+    s.n_zero = (size_t)(p - static_cast<char*>(base)) / 16;
+    return s;
 }
 
 // --- validation and access table ---------------------------------------------
-__global__ void fold_validate(const ExecArgs a, uint32_t* __restrict__ keys,
-                              uint32_t* __restrict__ vals, uint32_t* __restrict__ valid_flag,
-                              uint32_t none) {
-    __shared__ uint32_t skeys[32][64];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+// A lane group of G lanes per transaction (G the smallest of 8, 16, 32 that
+// holds max_ops; above 32 ops a lane takes two), U consecutive transactions
+// per group at once so that their headers and descriptors load together.
+// Every block takes one contiguous range of transactions.  Bound by the
+// stream of descriptors in and keys out, and by the shared-memory histogram
+// updates (one per op and pass).
+template <int G>
+__global__ void __launch_bounds__(256)
+fold_validate(const __grid_constant__ ExecArgs a, const FoldKeys f, uint32_t* __restrict__ keys,
+              uint32_t* work, uint32_t per_block) {
+    constexpr int GROUPS = 256 / G, U = G == 32 ? 2 : 4;
+    __shared__ DigitHist h[SORT_MAX_PASSES];
+    const int lane = threadIdx.x & 31, lig = lane & (G - 1), gbase = lane & ~(G - 1);
+    const uint32_t group = threadIdx.x / G;
+    const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << G) - 1u) << gbase;
+    clear_digits(h);
+    after_previous();
+    __syncthreads();
+    const bool tiled = work[DW_UNTILED] == 0;
+    uint64_t t_end = (uint64_t)(blockIdx.x + 1) * per_block;
+    if (t_end > a.n_txns) t_end = a.n_txns;
     unsigned invalid = 0;
-    for (uint32_t t = blockIdx.x * (blockDim.x >> 5) + wib; t < a.n_txns; t += warps) {
-        const gcc_txn tx = a.txns[t];
-        const uint32_t nops = tx.n_ops;
-        const uint64_t first = tx.first_op;
-        bool bad = nops > a.max_ops || nops > 64 || tx.type != GCC_TXN_KV || first + nops > a.n_ops;
-        if (!bad) {
-            for (uint32_t j = lane; j < nops; j += 32) {
-                const uint64_t d = a.ops[first + j];
-                skeys[wib][j] = d_key(d);
-                if (d_key(d) >= a.n_records || d_field(d) >= a.n_fields ||
-                    (d_kind(d) != GCC_OP_READ && d_kind(d) != GCC_OP_ADD))
-                    bad = true;
+    for (uint64_t t0 = (uint64_t)blockIdx.x * per_block; t0 < t_end; t0 += GROUPS * U) {
+        const uint64_t tb = t0 + group * U;
+        uint32_t first[U], nops[U];
+        uint64_t d[U];
+        bool bad[U], inside[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            gcc_txn tx{0u, 0, (uint16_t)GCC_TXN_KV};
+            if (tb + u < t_end) tx = a.txns[tb + u];
+            first[u] = tx.first_op;
+            nops[u] = tx.n_ops;
+            inside[u] = tb + u < t_end && (uint64_t)tx.first_op + tx.n_ops <= a.n_ops;
+            bad[u] = tx.n_ops > a.max_ops || tx.n_ops > 64 || tx.type != GCC_TXN_KV || !inside[u];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            d[u] = !bad[u] && lig < nops[u] ? a.ops[(uint64_t)first[u] + lig] : 0ull;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool has = !bad[u] && lig < nops[u];
+            bool wrong = false;
+            if (has)
+                wrong = d_key(d[u]) >= a.n_records || d_field(d[u]) >= a.n_fields ||
+                        (d_kind(d[u]) != GCC_OP_READ && d_kind(d[u]) != GCC_OP_ADD);
+            // equal keys among the group's lanes
+            const unsigned holders = __ballot_sync(0xffffffffu, has);
+            const unsigned peers = __match_any_sync(0xffffffffu, d_key(d[u]));
+            if (has && __popc(peers & holders & gmask) > 1) wrong = true;
+            uint64_t d2 = 0;
+            if constexpr (G == 32) {
+                if (!bad[u] && nops[u] > 32) {           // uniform over the warp
+                    const bool has2 = lig + 32 < nops[u];
+                    if (has2) {
+                        d2 = a.ops[(uint64_t)first[u] + 32 + lig];
+                        wrong = wrong || d_key(d2) >= a.n_records || d_field(d2) >= a.n_fields ||
+                                (d_kind(d2) != GCC_OP_READ && d_kind(d2) != GCC_OP_ADD);
+                    }
+                    const unsigned h2 = __ballot_sync(0xffffffffu, has2);
+                    const unsigned p2 = __match_any_sync(0xffffffffu, d_key(d2));
+                    if (has2 && __popc(p2 & h2) > 1) wrong = true;
+                    for (int i = 0; i < 32; ++i) {
+                        const uint32_t k = __shfl_sync(0xffffffffu, d_key(d[u]), i);
+                        if (has2 && k == d_key(d2)) wrong = true;
+                    }
+                }
+            }
+            const unsigned any = __ballot_sync(0xffffffffu, wrong);
+            const bool no = bad[u] || (any & gmask);
+            if (has) {
+                const uint64_t op = (uint64_t)first[u] + lig;
+                const uint32_t k = f.key(op, no ? f.n_slots : d_field(d[u]) * (uint32_t)a.n_records + d_key(d[u]),
+                                         !no && d_kind(d[u]) == GCC_OP_ADD);
+                keys[op] = k;
+                if (tiled) count_digits(h, k, f.bits, f.passes, f.digit_bits);
+            }
+            // the ops past the first G of a long or malformed transaction
+            if (inside[u] && (bad[u] || nops[u] > G)) {
+                for (uint32_t j = (bad[u] ? 0u : (uint32_t)G) + lig; j < nops[u]; j += G) {
+                    const uint64_t op = (uint64_t)first[u] + j;
+                    const uint32_t k = f.key(op, no ? f.n_slots : d_field(d2) * (uint32_t)a.n_records + d_key(d2),
+                                             !no && d_kind(d2) == GCC_OP_ADD);
+                    keys[op] = k;
+                    if (tiled) count_digits(h, k, f.bits, f.passes, f.digit_bits);
+                }
+            }
+            if (lig == 0 && tb + u < t_end) {
+                a.results[tb + u] = no ? gcc_txn_result{GCC_TXN_INVALID, 0u, ~0ull}
+                                       : gcc_txn_result{GCC_TXN_COMMITTED, 1u, tb + u};
+                invalid += no;
             }
         }
-        __syncwarp();
-        if (!__any_sync(0xffffffffu, bad)) {
-            for (uint32_t j = lane; j < nops; j += 32)
-                for (uint32_t i = 0; i < j; ++i)
-                    if (skeys[wib][i] == skeys[wib][j]) bad = true;
-        }
-        bad = __any_sync(0xffffffffu, bad);
-        if (first + nops <= a.n_ops) {
-            for (uint32_t j = lane; j < nops; j += 32) {
-                const uint64_t d = a.ops[first + j];
-                keys[first + j] = bad ? none : d_field(d) * (uint32_t)a.n_records + d_key(d);
-                vals[first + j] = (uint32_t)(first + j);
-            }
-        }
-        if (lane == 0) {
-            valid_flag[t] = bad ? 0u : 1u;
-            a.results[t] = bad ? gcc_txn_result{GCC_TXN_INVALID, 0u, ~0ull}
-                               : gcc_txn_result{GCC_TXN_COMMITTED, 1u, 0ull};
-            invalid += bad;
-        }
-        __syncwarp();
     }
-    if (lane == 0 && invalid) {
+    if (invalid) {
         atomicAdd(&a.st->invalid, (unsigned long long)invalid);
         atomicOr(&a.st->error, GCC_DEVERR_INVALID);
     }
+    flush_digits(h, work, keys, a.n_ops, f.bits, f.passes, f.digit_bits);
 }
 
-// Ops not covered by any transaction's range stay out of the access table.
-__global__ void fold_fill_none(uint32_t* __restrict__ keys, uint64_t n, uint32_t none) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) keys[i] = none;
-}
-
-// --- segmented scan ---------------------------------------------------------
-template <int FB>
-__device__ __forceinline__ Seg element(const ExecArgs& a, const uint32_t* sk, const uint32_t* sv,
-                                       uint64_t p, uint64_t n, uint32_t none) {
-    if (p >= n) return Seg{1u, Sum{0, 0}};
-    const uint32_t k = sk[p];
-    if (k == none) return Seg{1u, Sum{0, 0}};
-    const uint32_t head = (p == 0 || sk[p - 1] != k) ? 1u : 0u;
-    const uint32_t op = sv[p];
-    Sum v{0, 0};
-    if (d_kind(a.ops[op]) == GCC_OP_ADD) {
-        const ulonglong2 o = a.operands[op];
-        v = Sum{o.x, FB == 16 ? (o.y & 0xFFFFull) : 0ull};
-    }
-    return Seg{head, v};
-}
-
-// The same element from the cache fold_tile_totals filled: the op's delta,
-// stored in sorted order, so the second pass streams it instead of gathering
-// the op and its operand again.
-__device__ __forceinline__ Seg cached_element(const uint32_t* sk, const Sum* cache, uint64_t p,
-                                              uint64_t n, uint32_t none) {
-    if (p >= n) return Seg{1u, Sum{0, 0}};
-    const uint32_t k = sk[p];
-    if (k == none) return Seg{1u, Sum{0, 0}};
-    return Seg{(p == 0 || sk[p - 1] != k) ? 1u : 0u, cache[p]};
-}
-
-template <int FB>
-__global__ void __launch_bounds__(FB_THREADS)
-fold_tile_totals(const ExecArgs a, const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv,
-                 uint64_t n, uint32_t none, Seg* __restrict__ tile_tot, Sum* __restrict__ cache) {
-    __shared__ Seg warp_tot[33];
-    const uint64_t base = (uint64_t)blockIdx.x * FB_TILE + (uint64_t)threadIdx.x * FB_ITEMS;
-    Seg acc{0u, Sum{0, 0}};
-#pragma unroll
-    for (int i = 0; i < FB_ITEMS; ++i) {
-        const Seg e = element<FB>(a, sk, sv, base + i, n, none);
-        if (base + i < n) cache[base + i] = e.v;
-        acc = seg_combine(acc, e);
-    }
-    Seg total;
-    block_seg_exclusive(acc, warp_tot, &total);
-    if (threadIdx.x == 0) tile_tot[blockIdx.x] = total;
-}
-
-// Exclusive segmented scan of the tile totals (one block, running carry).
-__global__ void __launch_bounds__(FB_THREADS)
-fold_scan_tiles(Seg* __restrict__ tile_tot, uint32_t ntiles) {
-    __shared__ Seg warp_tot[33];
-    Seg carry{0u, Sum{0, 0}};
-    for (uint32_t base = 0; base < ntiles; base += FB_THREADS) {
-        const uint32_t i = base + threadIdx.x;
-        const Seg x = i < ntiles ? tile_tot[i] : Seg{0u, Sum{0, 0}};
-        Seg total;
-        const Seg ex = block_seg_exclusive(x, warp_tot, &total);
-        if (i < ntiles) tile_tot[i] = seg_combine(carry, ex);
-        carry = seg_combine(carry, total);
-    }
-}
-
+// --- fold -------------------------------------------------------------------
 template <int FB>
 __device__ __forceinline__ ulonglong2 slot_load(const ExecArgs& a, uint32_t slot) {
     const uint8_t* p = a.table + (uint64_t)slot * FB;
@@ -230,150 +238,250 @@ __device__ __forceinline__ ulonglong2 slot_plus(ulonglong2 v, Sum s) {
     return make_ulonglong2(v.x + s.lo, 0ull);
 }
 
-// Read values: initial slot value plus the exclusive prefix within the slot.
-// A slot whose accesses all lie in this tile also gets its final value here:
-// once the block's initial-value loads are done (the barrier), the slot's
-// last access writes initial + inclusive sum.  Slots whose accesses began in
-// an earlier tile are left to fold_finals, after every tile has loaded.
-template <int FB>
-__global__ void __launch_bounds__(FB_THREADS)
-fold_apply(const ExecArgs a, const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv,
-           uint64_t n, uint32_t none, const Seg* __restrict__ tile_carry,
-           const Sum* __restrict__ cache) {
-    __shared__ Seg warp_tot[33];
-    const uint64_t tile_base = (uint64_t)blockIdx.x * FB_TILE;
-    const uint64_t base = tile_base + (uint64_t)threadIdx.x * FB_ITEMS;
-    Seg e[FB_ITEMS];
-    Seg acc{0u, Sum{0, 0}};
+// Tile descriptor: x the sum's lane 0, y bits 0..15 its bytes 8-9, bits 62..63
+// the state.  TAIL: no slot's accesses begin in the tile, the sum is the whole
+// tile's and what comes before adds to it.  WHOLE: the sum from the beginning
+// of the slot whose accesses run on past the tile.
+constexpr uint64_t TAIL = 1ull << 62, WHOLE = 2ull << 62;
+
+// The sum of the accesses before `tile` to the slot that runs into it, by the
+// lanes of one warp, 32 predecessors at a time (usually one: nearly every tile
+// begins some slot).  Acquire loads: the caller may write that slot only after
+// every tile it runs through has read its initial value.
+__device__ __forceinline__ Sum fold_look_back(const ulonglong2* desc, int64_t tile, unsigned* err) {
+    const int lane = threadIdx.x & 31;
+    Sum sum{0, 0};
+    uint32_t spins = 0;
+    for (int64_t p = tile - 1; p >= 0;) {
+        ulonglong2 w = make_ulonglong2(0ull, WHOLE);
+        if (p - lane >= 0) w = ld128_acquire(desc + (p - lane));
+        const unsigned whole = __ballot_sync(0xffffffffu, w.y >= WHOLE);
+        const unsigned none = __ballot_sync(0xffffffffu, w.y == 0);
+        const int upto = whole ? __ffs(whole) - 1 : 31;             // last lane that counts
+        const unsigned need = upto == 31 ? 0xffffffffu : (2u << upto) - 1u;
+        if (none & need) {
+            if (++spins > DET_SPIN_MAX) {
+                if (lane == 0) atomicOr(err, GCC_DEVERR_WAIT_BUDGET);
+                return sum;
+            }
+            continue;
+        }
+        uint64_t lo = lane <= upto ? w.x : 0ull;
+        uint32_t hi = lane <= upto ? (uint32_t)w.y & 0xFFFFu : 0u;
 #pragma unroll
-    for (int i = 0; i < FB_ITEMS; ++i) {
-        e[i] = cached_element(sk, cache, base + i, n, none);
-        acc = seg_combine(acc, e[i]);
+        for (int o = 16; o > 0; o >>= 1) {
+            lo += __shfl_xor_sync(0xffffffffu, lo, o);
+            hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        }
+        sum = sum_add(sum, Sum{lo, hi});
+        if (whole) break;
+        p -= 32;
     }
-    Seg run = seg_combine(tile_carry[blockIdx.x], block_seg_exclusive(acc, warp_tot, nullptr));
-    const uint32_t before = tile_base > 0 ? sk[tile_base - 1] : none;   // key entering the tile
-    ulonglong2 fin[FB_ITEMS];
-    bool last[FB_ITEMS];
+    return sum;
+}
+
+// One tile of sorted accesses: an access reads its slot's initial value
+// plus the sum of the deltas before it, the last access of a slot stores the
+// final value.  Within the tile every initial value is read before the block
+// barrier and stored after it; a slot that runs through several tiles is stored
+// by the last of them, after it has acquired the descriptors of the others,
+// which they publish (release) behind that barrier.
+// Bound by the table's random DRAM accesses (a load and, for a changed slot,
+// a write-back each; the part sustains about 39 G of them a second): 2^21 ops
+// over 2.5 GiB take 0.1 ms.  One kernel instead of three (tile totals, tile
+// scan, apply, and a fourth for slots that cross tiles) removes a 16-byte
+// delta per op written and read back; the four took 1.46 ms for 2^24 ops, the
+// eight launches of this one 0.83 ms.
+template <int FB>
+__global__ void __launch_bounds__(FT_THREADS, 4)
+fold_tiles(const __grid_constant__ ExecArgs a, const FoldKeys f, const uint32_t* __restrict__ sk,
+           const uint32_t* __restrict__ sv, uint64_t op0, uint32_t c0, uint32_t c1,
+           uint32_t* ticket, ulonglong2* desc) {
+    constexpr int ITEMS = FT_ITEMS<FB>;
+    __shared__ uint32_t s_tile;
+    __shared__ uint64_t s_lo[FT_WARPS];
+    __shared__ uint32_t s_hi[FT_WARPS];        // bit 31: the warp begins a slot
+    __shared__ Sum s_carry;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    after_previous();
+    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+    __syncthreads();
+    const uint32_t tile = s_tile;
+    const uint32_t base = c0 + tile * FT_TILE<FB> + threadIdx.x * ITEMS;
+    uint32_t k[ITEMS], v[ITEMS];
+    if (base + ITEMS <= c1) {
+        if constexpr (ITEMS == 4) {
+            const uint4 x = *reinterpret_cast<const uint4*>(sk + base);
+            const uint4 y = *reinterpret_cast<const uint4*>(sv + base);
+            k[0] = x.x; k[1] = x.y; k[2] = x.z; k[3] = x.w;
+            v[0] = y.x; v[1] = y.y; v[2] = y.z; v[3] = y.w;
+        } else {
+            const uint2 x = *reinterpret_cast<const uint2*>(sk + base);
+            const uint2 y = *reinterpret_cast<const uint2*>(sv + base);
+            k[0] = x.x; k[1] = x.y;
+            v[0] = y.x; v[1] = y.y;
+        }
+    } else {
 #pragma unroll
-    for (int i = 0; i < FB_ITEMS; ++i) {
-        const uint64_t p = base + i;
-        const Sum prefix = e[i].head ? Sum{0, 0} : run.v;
-        last[i] = false;
-        if (p < n && sk[p] != none) {
-            const uint32_t k = sk[p];
-            const uint32_t op = sv[p];
-            const ulonglong2 init = slot_load<FB>(a, k);
-            const ulonglong2 rd = slot_plus<FB>(init, prefix);
-            a.reads[op] = rd;
-            if ((p + 1 >= n || sk[p + 1] != k) && k != before) {
-                fin[i] = slot_plus<FB>(rd, e[i].v);
-                last[i] = fin[i].x != init.x || fin[i].y != init.y;   // skip unchanged slots
+        for (int i = 0; i < ITEMS; ++i) {
+            k[i] = base + i < c1 ? sk[base + i] : 0u;
+            v[i] = base + i < c1 ? sv[base + i] : 0u;
+        }
+    }
+    // the keys around the thread's own
+    uint32_t prev = __shfl_up_sync(0xffffffffu, k[ITEMS - 1], 1);
+    uint32_t next = __shfl_down_sync(0xffffffffu, k[0], 1);
+    if (lane == 0) prev = base > c0 && base < c1 ? sk[base - 1] : 0u;
+    if (lane == 31) next = base + ITEMS < c1 ? sk[base + ITEMS] : 0u;
+    uint32_t head = 0, live = 0;               // bit per item
+    ulonglong2 init[ITEMS];
+    Sum dl[ITEMS];
+    uint32_t seen = 0;
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const bool in = base + i < c1 && f.slot(k[i]) < f.n_slots && f.op(op0, v[i]) < a.n_ops;
+        live |= in ? 1u << i : 0u;
+        if (!in || (i == 0 ? base == c0 || prev != k[0] : k[i - 1] != k[i])) head |= 1u << i;
+        dl[i] = Sum{0, 0};
+        init[i] = make_ulonglong2(0ull, 0ull);
+        if (in) init[i] = slot_load<FB>(a, f.slot(k[i]));
+    }
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i)
+        if ((live >> i & 1) && (f.flagged ? v[i] >> 31 : d_kind(a.ops[f.op(op0, v[i])]) == GCC_OP_ADD)) {
+            const ulonglong2 o = a.operands[f.op(op0, v[i])];
+            dl[i] = Sum{o.x, FB == 16 ? (uint32_t)o.y & 0xFFFFu : 0u};
+        }
+    // within the thread
+    Sum run{0, 0};
+    const bool any = head != 0;
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        if (head >> i & 1) run = Sum{0, 0};
+        run = sum_add(run, dl[i]);
+        seen ^= (uint32_t)init[i].x;
+    }
+    // within the warp: inclusive sums since the last lane that begins a slot
+    const unsigned heads = __ballot_sync(0xffffffffu, any);
+    const unsigned upto = heads & (0xffffffffu >> (31 - lane));
+    const int start = upto ? 31 - __clz(upto) : 0;
+    Sum inc = run;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t lo = __shfl_up_sync(0xffffffffu, inc.lo, o);
+        const uint32_t hi = FB == 16 ? __shfl_up_sync(0xffffffffu, inc.hi, o) : 0u;
+        if (lane - o >= start) inc = sum_add(inc, Sum{lo, hi});
+    }
+    Sum carry;                                 // what precedes the thread, in the warp
+    carry.lo = __shfl_up_sync(0xffffffffu, inc.lo, 1);
+    carry.hi = FB == 16 ? __shfl_up_sync(0xffffffffu, inc.hi, 1) : 0u;
+    if (lane == 0) carry = Sum{0, 0};
+    if (lane == 31) {
+        s_lo[warp] = inc.lo;
+        s_hi[warp] = inc.hi | (heads ? 0x80000000u : 0u);
+    }
+    // the barrier takes a predicate computed from the initial values, so every
+    // one of this tile has arrived before any thread passes it
+    __syncthreads_or(seen == 0x9E3779B9u);
+    const bool runs_in = !(head & 1);          // thread 0: the tile continues a slot
+    if (warp == 0) {
+        Sum tot{0, 0};
+        bool begins = false;
+#pragma unroll
+        for (int w = 0; w < FT_WARPS; ++w) {
+            if (s_hi[w] >> 31) { tot = Sum{0, 0}; begins = true; }
+            tot = sum_add(tot, Sum{s_lo[w], s_hi[w] & 0xFFFFu});
+        }
+        const bool whole = begins || tile == 0;
+        if (lane == 0) st128_release(desc + tile, make_ulonglong2(tot.lo, tot.hi | (whole ? WHOLE : TAIL)));
+        Sum before{0, 0};
+        if (__shfl_sync(0xffffffffu, runs_in, 0)) {
+            before = fold_look_back(desc, tile, &a.st->error);
+            if (!whole && lane == 0) {
+                const Sum all = sum_add(before, tot);
+                st128_release(desc + tile, make_ulonglong2(all.lo, all.hi | WHOLE));
             }
         }
-        run = seg_combine(run, e[i]);
+        if (lane == 0) s_carry = before;
     }
-    __syncthreads();                      // every initial value of this tile has been read
+    __syncthreads();
+    if (!(heads & (0xffffffffu >> (31 - lane)) & ~(1u << lane))) {   // no lane before begins a slot
+        bool open = true;
+        for (int w = warp - 1; w >= 0 && open; --w) {
+            carry = sum_add(carry, Sum{s_lo[w], s_hi[w] & 0xFFFFu});
+            open = !(s_hi[w] >> 31);
+        }
+        if (open) carry = sum_add(carry, s_carry);
+    }
 #pragma unroll
-    for (int i = 0; i < FB_ITEMS; ++i) {
-        if (!last[i]) continue;
-        uint8_t* dst = a.table + (uint64_t)sk[base + i] * FB;
-        if (FB == 16) *reinterpret_cast<ulonglong2*>(dst) = fin[i];
-        else *reinterpret_cast<uint64_t*>(dst) = fin[i].x;
+    for (int i = 0; i < ITEMS; ++i) {
+        if (head >> i & 1) carry = Sum{0, 0};
+        if (!(live >> i & 1)) continue;
+        a.reads[f.op(op0, v[i])] = slot_plus<FB>(init[i], carry);
+        carry = sum_add(carry, dl[i]);
+        const bool last = base + i + 1 >= c1 || (i + 1 < ITEMS ? k[(i + 1) % ITEMS] : next) != k[i];
+        if (last && (carry.lo | carry.hi)) {                     // unchanged slots are not stored
+            const ulonglong2 fin = slot_plus<FB>(init[i], carry);
+            uint8_t* dst = a.table + (uint64_t)f.slot(k[i]) * FB;
+            if (FB == 16) *reinterpret_cast<ulonglong2*>(dst) = fin;
+            else *reinterpret_cast<uint64_t*>(dst) = fin.x;
+        }
     }
 }
-
-// The last access of each slot whose accesses began in an earlier tile
-// installs the final value (the others were installed by fold_apply).
-template <int FB>
-__global__ void fold_finals(const ExecArgs a, const uint32_t* __restrict__ sk,
-                            const uint32_t* __restrict__ sv, uint64_t n, uint32_t none) {
-    const uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const uint32_t k = sk[p];
-    if (k == none || (p + 1 < n && sk[p + 1] == k)) return;
-    const uint64_t tile_base = p / FB_TILE * FB_TILE;
-    if (tile_base == 0 || sk[tile_base - 1] != k) return;     // installed by fold_apply
-    const uint32_t op = sv[p];
-    ulonglong2 v = a.reads[op];                   // initial value + every earlier delta
-    if (d_kind(a.ops[op]) == GCC_OP_ADD) {
-        const ulonglong2 o = a.operands[op];
-        v = slot_plus<FB>(v, Sum{o.x, FB == 16 ? (o.y & 0xFFFFull) : 0ull});
-    }
-    // only this thread touches the slot now; skip slots that did not change
-    const ulonglong2 cur = slot_load<FB>(a, k);
-    if (cur.x == v.x && cur.y == v.y) return;
-    uint8_t* dst = a.table + (uint64_t)k * FB;
-    if (FB == 16) *reinterpret_cast<ulonglong2*>(dst) = v;
-    else *reinterpret_cast<uint64_t*>(dst) = v.x;
-}
-
-// commit order = rank among valid transactions; counts the commits
-__global__ void fold_ranks(const ExecArgs a, const uint32_t* __restrict__ rank, uint32_t n) {
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    if (a.results[t].status == GCC_TXN_COMMITTED) a.results[t].commit_order = rank[t];
-}
-
-__global__ void fold_count(const ExecArgs a, const uint32_t* __restrict__ rank,
-                           const uint32_t* __restrict__ flag, uint32_t n) {
-    if (n) {
-        a.st->committed = rank[n - 1] + flag[n - 1];
-        a.st->max_attempts = a.st->committed ? 1ull : 0ull;
-    }
-}
-
-inline unsigned blocks_for(uint64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
 template <int FB>
-cudaError_t fold_run(const ExecArgs& a, SortScratch& s, uint32_t* scan_tmp, uint32_t* flags,
-                     void* seg_tmp, cudaStream_t st) {
+cudaError_t fold_run(const ExecArgs& a, SortScratch& s, void* scratch, uint32_t& launches, cudaStream_t st) {
     const uint64_t n = a.n_ops;
-    const uint64_t n_slots = (uint64_t)a.n_fields * a.n_records;
-    const uint32_t none = (uint32_t)n_slots;               // sorts after every slot
-    int bits = 0;
-    for (uint64_t v = n_slots; v; v >>= 1) ++bits;
-    if (n) fold_fill_none<<<blocks_for(n, 256), 256, 0, st>>>(s.k0, n, none);
-    if (a.n_txns) {
-        const int warps_per_block = 8;
-        const unsigned grid = std::min<unsigned>(blocks_for(a.n_txns, warps_per_block), 152u * 16u);
-        fold_validate<<<grid, warps_per_block * 32, 0, st>>>(a, s.k0, s.v0, flags, none);
+    const FoldKeys f = fold_keys((uint64_t)a.n_fields * a.n_records, n);
+    const FoldScratch sc = fold_scratch(scratch, n, a.n_txns);
+    const bool one_sort = n <= (1ull << SORT_LOG2);
+    const size_t n_zero = one_sort ? (SORT_DESC - SORT_HIST + sort_desc_words(n)) / 4 : 0;
+    const uint64_t most = std::max<uint64_t>(std::max<uint64_t>(n_zero, sc.n_zero), a.n_txns);
+    const unsigned grid0 = std::min<unsigned>(std::max<unsigned>(blocks_for(most, 256), 1u), 608u);
+    cudaError_t e = launch_after(det_begin<FoldKeys>, grid0, 256, st, a, s.work,
+                                 reinterpret_cast<ulonglong2*>(s.work + SORT_HIST), n_zero, sc.zero,
+                                 sc.n_zero, s.k0, f);
+    launches += 1;
+    if (e != cudaSuccess || a.n_txns == 0) return e;
+    const int G = a.max_ops <= 8 ? 8 : a.max_ops <= 16 ? 16 : 32;
+    const uint32_t step = G == 8 ? 128 : G == 16 ? 64 : 16;
+    const uint32_t steps = blocks_for(a.n_txns, (int)step);
+    const uint32_t per_block = (uint32_t)blocks_for(steps, 152 * 6) * step;
+    const unsigned grid1 = blocks_for(a.n_txns, (int)per_block);
+    auto validate = G == 8 ? fold_validate<8> : G == 16 ? fold_validate<16> : fold_validate<32>;
+    e = launch_after(validate, grid1, 256, st, a, f, s.k0, s.work, per_block);
+    launches += 1;
+    for (uint64_t o0 = 0; o0 < n && e == cudaSuccess; o0 += 1ull << SORT_LOG2) {
+        const uint32_t m = (uint32_t)std::min<uint64_t>(n - o0, 1ull << SORT_LOG2);
+        uint32_t *sk = nullptr, *sv = nullptr;
+        e = radix_sort_positions(s, s.k0 + o0, m, f.bits, f.flagged != 0, one_sort, &sk, &sv, st);
+        launches += f.passes + (one_sort ? 0 : 1);
+        for (uint32_t c0 = 0; c0 < m && e == cudaSuccess;) {
+            const uint32_t len = f.chunk_log2 >= 31 ? m : std::min<uint32_t>(m - c0, 1u << f.chunk_log2);
+            const uint64_t at = o0 + c0;
+            e = launch_after(fold_tiles<FB>, blocks_for(len, FT_TILE<FB>), FT_THREADS, st, a, f, sk, sv, o0, c0,
+                             c0 + len, sc.tickets + (at >> CHUNK_LOG2), sc.tile_desc + at / FT_TILE<FB>);
+            launches += 1;
+            c0 += len;
+        }
     }
-    uint32_t *sk = s.k0, *sv = s.v0;
-    if (n) {
-        cudaError_t e = radix_sort_pairs(s, n, bits, &sk, &sv, st);
-        if (e != cudaSuccess) return e;
-        const uint32_t ntiles = (uint32_t)((n + FB_TILE - 1) / FB_TILE);
-        Seg* tiles = static_cast<Seg*>(seg_tmp);
-        Sum* cache = reinterpret_cast<Sum*>(static_cast<char*>(seg_tmp) + fold_carry_bytes(n));
-        fold_tile_totals<FB><<<ntiles, FB_THREADS, 0, st>>>(a, sk, sv, n, none, tiles, cache);
-        fold_scan_tiles<<<1, FB_THREADS, 0, st>>>(tiles, ntiles);
-        fold_apply<FB><<<ntiles, FB_THREADS, 0, st>>>(a, sk, sv, n, none, tiles, cache);
-        fold_finals<FB><<<blocks_for(n, 256), 256, 0, st>>>(a, sk, sv, n, none);
-    }
-    if (a.n_txns) {
-        // dense commit order: exclusive count of valid transactions before each
-        uint32_t* rank = flags + a.n_txns;
-        cudaError_t e = cudaMemcpyAsync(rank, flags, (size_t)a.n_txns * 4,
-                                        cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
-        e = exclusive_scan_u32(rank, a.n_txns, scan_tmp, st);
-        if (e != cudaSuccess) return e;
-        fold_ranks<<<blocks_for(a.n_txns, 256), 256, 0, st>>>(a, rank, a.n_txns);
-        fold_count<<<1, 1, 0, st>>>(a, rank, flags, a.n_txns);
-    }
-    return cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    launches += 1;
+    return launch_after(det_finish, std::min<unsigned>(blocks_for(a.n_txns, RANK_TILE), 152u), 1024, st, a,
+                        s.work, sc.rank_desc);
 }
 
 }  // namespace
 
-size_t fold_seg_bytes(size_t max_ops) {
-    return fold_carry_bytes(max_ops) + max_ops * sizeof(Sum);
+// (the version store of an MVCC batch shares this scratch: one 16-byte value per op)
+size_t fold_seg_bytes(size_t max_ops, size_t max_txns) {
+    return std::max<size_t>(max_ops * 16, fold_scratch(nullptr, max_ops, max_txns).n_zero * 16);
 }
 
-cudaError_t det_fold_kv(const ExecArgs& a, uint32_t field_bytes, SortScratch& s,
-                        uint32_t* scan_tmp, uint32_t* flags, void* seg_tmp, cudaStream_t st) {
-    return field_bytes == 16 ? fold_run<16>(a, s, scan_tmp, flags, seg_tmp, st)
-                             : fold_run<8>(a, s, scan_tmp, flags, seg_tmp, st);
+cudaError_t det_fold_kv(const ExecArgs& a, uint32_t field_bytes, SortScratch& s, void* scratch,
+                        uint32_t& launches, cudaStream_t st) {
+    return field_bytes == 16 ? fold_run<16>(a, s, scratch, launches, st)
+                             : fold_run<8>(a, s, scratch, launches, st);
 }
 
 }  // namespace gcc

@@ -115,6 +115,13 @@ __device__ __forceinline__ ulonglong2 ld128_acquire(const void* p) {
         : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ void st128_release(void* p, ulonglong2 v) {
+    asm volatile(
+        "{\n\t.reg .b128 d;\n\t"
+        "mov.b128 d, {%1, %2};\n\t"
+        "st.release.gpu.global.b128 [%0], d;\n\t}"
+        ::"l"(p), "l"(v.x), "l"(v.y) : "memory");
+}
 __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* p) {
     uint32_t v;
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -269,6 +276,33 @@ __host__ __device__ __forceinline__ uint32_t cc_record(uint64_t d, int schema, u
 }
 
 // ---------------------------------------------------------------------------
+// dependent launches
+// ---------------------------------------------------------------------------
+// A kernel launched with launch_after may be scheduled while its predecessor
+// in the stream drains; it calls after_previous() before it touches memory,
+// which waits until the predecessor has completed and its writes are visible,
+// and lets its own successor be scheduled in turn.  A chain of short kernels
+// then costs little more than its kernels.
+__device__ __forceinline__ void after_previous() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+inline cudaError_t launch_after(void (*k)(P...), unsigned grid, unsigned block, cudaStream_t st,
+                                A&&... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(block);
+    c.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // kernel arguments
 // ---------------------------------------------------------------------------
 struct ExecArgs {
@@ -362,15 +396,63 @@ cudaError_t launch_batch_begin(BatchState* st, DbState* dbs, gcc_scheme scheme,
 
 // Stable LSD radix sort of (key, value) u32 pairs on the low `bits` bits.
 // Sorted output lands in (*keys_out, *vals_out), one of the two buffer pairs.
+//
+// `work` (sort_work_words(max_items) words) holds the tile tickets, the digit
+// histograms of every pass and two descriptor areas that the passes use in
+// turn (order.cu).
 struct SortScratch {
     uint32_t *k0, *v0, *k1, *v1;
-    uint32_t* hist;               // 256 * max_tiles
-    uint32_t* totals;             // 256
+    uint32_t* work;
     size_t max_items;
+    unsigned* err = nullptr;      // GCC_DEVERR_* word a bounded wait reports into
 };
-size_t sort_max_tiles(size_t n);
+// Word layout of `work`: pass tickets, then words of the deterministic passes
+// (det_common.cuh), then one 256-bin histogram per pass, then the descriptors.
+constexpr int SORT_MAX_PASSES = 4;
+constexpr size_t SORT_HIST = 64;
+constexpr size_t SORT_DESC = SORT_HIST + SORT_MAX_PASSES * 256;
+// Items per tile: few enough per thread that a small sort still covers the
+// SMs, many for the large ones (order.cu gives the measurements).
+constexpr int SORT_BLOCK = 256;
+constexpr int SORT_ITEMS_SMALL = 4, SORT_ITEMS_LARGE = 16;
+constexpr size_t SORT_SMALL = size_t(1) << 19;
+constexpr size_t sort_tiles(size_t n) {
+    const size_t tile = SORT_BLOCK * (n <= SORT_SMALL ? SORT_ITEMS_SMALL : SORT_ITEMS_LARGE);
+    return (n + tile - 1) / tile;
+}
+// Words of one descriptor area: 256 per tile, 64-bit where a digit's count may
+// pass 30 bits.  Any n up to max_items must fit.
+constexpr size_t sort_desc_words(size_t n) {
+    return sort_tiles(n) * 256 * (n >= (size_t(1) << 30) ? 2 : 1);
+}
+constexpr size_t sort_work_words(size_t max_items) {
+    const size_t a = sort_desc_words(max_items);
+    const size_t b = sort_desc_words(max_items < SORT_SMALL ? max_items : SORT_SMALL);
+    return SORT_DESC + 2 * (a > b ? a : b);
+}
+struct SortPlan {                 // digits of a sort on the low `bits` bits
+    int passes, digit_bits;
+    int width(int bits, int p) const {
+        const int left = bits - p * digit_bits;
+        return left < digit_bits ? left : digit_bits;
+    }
+};
+inline SortPlan sort_plan(int bits) {
+    SortPlan s;
+    s.passes = (bits + 7) / 8;
+    s.digit_bits = s.passes ? (bits + s.passes - 1) / s.passes : 0;
+    return s;
+}
 cudaError_t radix_sort_pairs(SortScratch& s, size_t n, int bits, uint32_t** keys_out,
                              uint32_t** vals_out, cudaStream_t st);
+int radix_sort_launches(int bits);
+// The same with keys in `keys` (used as the first key buffer) and values =
+// positions; with `flagged` bit 31 of a key, outside the sorted bits, moves to
+// bit 31 of its value.  `prepared`: the kernels that made the keys left their
+// histograms in `work`, with its tickets and its first descriptor area zeroed.
+cudaError_t radix_sort_positions(SortScratch& s, uint32_t* keys, size_t n, int bits, bool flagged,
+                                 bool prepared, uint32_t** keys_out, uint32_t** vals_out,
+                                 cudaStream_t st);
 
 // Exclusive prefix sum of u32 (in place), with `tmp` of >= scan_tmp_words(n).
 size_t scan_tmp_words(size_t n);
@@ -391,9 +473,12 @@ cudaError_t det_prepare(const ExecArgs& a, SortScratch& s, uint32_t* scan_tmp, i
 // Record `msg` as this thread's gcc_last_error() and return `s`.
 gcc_status set_error(gcc_status s, const char* msg);
 
-// Deterministic scheme on a key-value batch by segmented prefix sums; `flags`
-// holds 2 * n_txns words, `seg_tmp` fold_seg_bytes(n_ops) bytes.
-size_t fold_seg_bytes(size_t max_ops);
+// Deterministic scheme on a key-value batch by segmented prefix sums; `scratch`
+// holds fold_seg_bytes(max_batch_ops, max_batch_txns) bytes; adds the kernels
+// it launches to `launches`.  Begins the batch itself (no launch_batch_begin).
+size_t fold_seg_bytes(size_t max_ops, size_t max_txns);
+cudaError_t det_fold_kv(const ExecArgs& a, uint32_t field_bytes, SortScratch& s, void* scratch,
+                        uint32_t& launches, cudaStream_t st);
 // Deterministic order-entry batch: each record's accesses applied in id order
 // by one warp over the sorted access table (reads, final records, NewOrder
 // inserts, results, dense ranks, batch counters).  `flags` holds 2 * n_txns
@@ -401,8 +486,6 @@ size_t fold_seg_bytes(size_t max_ops);
 cudaError_t det_serial_oe(const ExecArgs& a, SortScratch& s, uint32_t* scan_tmp, uint32_t* flags,
                           uint32_t* heads, int key_bits, int sm_count, cudaStream_t st);
 int det_serial_oe_launches(int key_bits);
-cudaError_t det_fold_kv(const ExecArgs& a, uint32_t field_bytes, SortScratch& s,
-                        uint32_t* scan_tmp, uint32_t* flags, void* seg_tmp, cudaStream_t st);
 
 // OCC / TO: replace raw commit timestamps by dense ranks 0..committed-1.
 cudaError_t densify_commit_order(const ExecArgs& a, SortScratch& s, cudaStream_t st);

@@ -299,8 +299,7 @@ void free_plan(gcc_multi_plan* pl) {
     cudaFree(pl->sort.v0);
     cudaFree(pl->sort.k1);
     cudaFree(pl->sort.v1);
-    cudaFree(pl->sort.hist);
-    cudaFree(pl->sort.totals);
+    cudaFree(pl->sort.work);
     for (cudaStream_t s : pl->side)
         if (s) { cudaStreamSynchronize(s); cudaStreamDestroy(s); }
     for (cudaEvent_t e : pl->ev)
@@ -325,13 +324,7 @@ gcc_status enqueue_det(gcc_multi_plan* pl, cudaStream_t st) {
     for (uint32_t i = 0; e == cudaSuccess && i < pl->n; ++i) {
         gcc_db* db = pl->dbs[i];
         cudaStream_t s = pl->side[i % k];
-        e = launch_batch_begin(db->st, db->dbs, GCC_DET, s);
-        if (e == cudaSuccess)
-            e = det_fold_kv(pl->h_args[i], pl->field_bytes, db->sort, db->scan_tmp, db->fold_flags,
-                            db->fold_seg, s);
-        int bits = 0;
-        for (uint64_t v = (uint64_t)db->d.n_fields * db->d.n_records; v; v >>= 1) ++bits;
-        launches += 1 + 2 + 3 * ((bits + 7) / 8) + 4 + 1 + 3 + 2;
+        e = det_fold_kv(pl->h_args[i], pl->field_bytes, db->sort, db->fold_seg, launches, s);
     }
     for (uint32_t j = 0; e == cudaSuccess && j < k; ++j) {
         e = cudaEventRecord(pl->ev[1 + j], pl->side[j]);
@@ -391,12 +384,12 @@ gcc_status enqueue(gcc_multi_plan* pl, cudaStream_t st) {
                     pl->d_args, pl->d_prefix, pl->n, pl->total, pass, pl->sort.k0, pl->sort.v0);
                 e = radix_sort_pairs(pl->sort, pl->total, 32, &sk, &sv, st);
             }
-            launches += 3 * (1 + 12);
+            launches += 3 * (1 + radix_sort_launches(32));
         } else {
             multi_rank_keys<<<blocks_for(pl->total, 256), 256, 0, st>>>(pl->d_args, pl->d_prefix, pl->n,
                                                                      pl->total, pl->sort.k0, pl->sort.v0);
             e = radix_sort_pairs(pl->sort, pl->total, 32, &sk, &sv, st);   // by timestamp
-            launches += 1 + 12;
+            launches += 1 + radix_sort_launches(32);
         }
         if (e == cudaSuccess) {
             multi_batch_keys<<<blocks_for(pl->total, 256), 256, 0, st>>>(pl->d_prefix, pl->n, pl->total,
@@ -407,7 +400,7 @@ gcc_status enqueue(gcc_multi_plan* pl, cudaStream_t st) {
         if (e == cudaSuccess)
             multi_ranks<<<blocks_for(pl->total, 256), 256, 0, st>>>(pl->d_args, pl->d_prefix, pl->n,
                                                                  pl->total, sv);
-        launches += 1 + 3 + 1;
+        launches += 1 + radix_sort_launches(8) + 1;
     }
     if (e == cudaSuccess) {
         multi_end<<<1, 256, 0, st>>>(pl->d_own, pl->n, pl->d_ms);
@@ -483,10 +476,10 @@ gcc_status gcc_multi_plan_create(gcc_scheme scheme, const gcc_multi_batch* b, ui
         !alloc((void**)&pl->d_ms, sizeof(gcc::MultiState)) ||
         !alloc((void**)&pl->sort.k0, items * 4) || !alloc((void**)&pl->sort.v0, items * 4) ||
         !alloc((void**)&pl->sort.k1, items * 4) || !alloc((void**)&pl->sort.v1, items * 4) ||
-        !alloc((void**)&pl->sort.hist, gcc::sort_max_tiles(items) * 256 * 4) ||
-        !alloc((void**)&pl->sort.totals, 256 * 4))
+        !alloc((void**)&pl->sort.work, gcc::sort_work_words(items) * 4))
         return bail(fail(GCC_ERR_NOMEM, "cannot allocate the plan"));
     pl->sort.max_items = items;
+    pl->sort.err = &b[0].db->st->error;      // any of the plan's batches: a sort serves them all
 
     std::vector<gcc::ExecArgs> args(n);
     std::vector<gcc::DbState*> own(n);
@@ -540,6 +533,7 @@ gcc_status gcc_multi_plan_create(gcc_scheme scheme, const gcc_multi_batch* b, ui
             // the database's own scratch and staging limit, as a plain launch
             a.max_ops = db->d.max_ops_per_txn;
             a.need = db->need;
+            a.dbs = db->dbs;
             a.order_key_uses_base = 0;
             continue;                    // control words are not used
         }

@@ -20,15 +20,13 @@ constexpr uint32_t NA_MAX = 65536;   // records, ops and transactions per call
 
 // Byte layout of the static scratch (each piece 256-byte aligned).
 constexpr size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
-constexpr size_t NA_TILES = (NA_MAX + 2047) / 2048;     // radix-sort tiles (of 2048 items or more)
 constexpr size_t OFF_META = 0;
 constexpr size_t OFF_K0 = OFF_META + align256(NA_MAX * 8);
 constexpr size_t OFF_V0 = OFF_K0 + align256(NA_MAX * 4);
 constexpr size_t OFF_K1 = OFF_V0 + align256(NA_MAX * 4);
 constexpr size_t OFF_V1 = OFF_K1 + align256(NA_MAX * 4);
-constexpr size_t OFF_HIST = OFF_V1 + align256(NA_MAX * 4);
-constexpr size_t OFF_TOTALS = OFF_HIST + align256(NA_TILES * 256 * 4);
-constexpr size_t OFF_SCAN = OFF_TOTALS + align256(256 * 4);
+constexpr size_t OFF_WORK = OFF_V1 + align256(NA_MAX * 4);
+constexpr size_t OFF_SCAN = OFF_WORK + align256(gcc::sort_work_words(NA_MAX) * 4);
 constexpr size_t OFF_NEED = OFF_SCAN + align256(64 * 4);
 constexpr size_t OFF_STATE = OFF_NEED + align256(NA_MAX * 4);
 constexpr size_t OFF_DBSTATE = OFF_STATE + align256(sizeof(gcc::BatchState));
@@ -99,8 +97,8 @@ gcc_status gcc_det_execute_noalloc(void* d_table, uint32_t n_records, uint32_t n
     sort.v0 = reinterpret_cast<uint32_t*>(base + OFF_V0);
     sort.k1 = reinterpret_cast<uint32_t*>(base + OFF_K1);
     sort.v1 = reinterpret_cast<uint32_t*>(base + OFF_V1);
-    sort.hist = reinterpret_cast<uint32_t*>(base + OFF_HIST);
-    sort.totals = reinterpret_cast<uint32_t*>(base + OFF_TOTALS);
+    sort.work = reinterpret_cast<uint32_t*>(base + OFF_WORK);
+    sort.err = &reinterpret_cast<gcc::BatchState*>(base + OFF_STATE)->error;
     sort.max_items = NA_MAX;
 
     gcc::ExecArgs a{};

@@ -79,7 +79,7 @@ __global__ void unit_links(const uint32_t* __restrict__ sk, const uint32_t* __re
 uint32_t occ_form_units_launches(uint64_t n_records) {
     int bits = 0;
     for (uint64_t v = n_records; v; v >>= 1) ++bits;
-    return 1 + 1 + 1 + 3 * (uint32_t)((bits + 7) / 8) + 1;
+    return 1 + 1 + 1 + (uint32_t)radix_sort_launches(bits) + 1;
 }
 
 cudaError_t occ_form_units(const ExecArgs& a, uint32_t* cnt, SortScratch& s, uint32_t* link,

@@ -19,9 +19,7 @@
 namespace gcc {
 namespace {
 
-constexpr int RS_BLOCK = 256;
-constexpr int RS_CHUNKS = 8;
-constexpr int RS_TILE = RS_BLOCK * RS_CHUNKS;
+constexpr int RS_BLOCK = SORT_BLOCK;
 constexpr int RS_WARPS = RS_BLOCK / 32;
 
 __device__ __forceinline__ unsigned lt_mask() {
@@ -60,110 +58,244 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* w
 }
 
 // --- radix sort --------------------------------------------------------------
-__global__ void rs_hist(const uint32_t* __restrict__ keys, size_t n, int shift,
-                        uint32_t* __restrict__ hist, uint32_t ntiles) {
-    __shared__ uint32_t h[256];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const size_t base = (size_t)blockIdx.x * RS_TILE;
-    for (int c = 0; c < RS_CHUNKS; ++c) {
-        const size_t i = base + (size_t)c * RS_BLOCK + threadIdx.x;
-        const uint32_t dg = i < n ? (keys[i] >> shift) & 255u : 256u;
-        const unsigned peers = __match_any_sync(0xffffffffu, dg);
-        if (dg < 256u && (peers & lt_mask()) == 0) atomicAdd(&h[dg], __popc(peers));
+// One kernel per pass.  The digit histograms of every pass are taken up front
+// in one read of the keys, so a pass knows where each digit's run starts; what
+// a tile still needs is the number of each digit's items in the tiles before
+// it, which it gets by looking back: every tile publishes its own counts at
+// once, sums its predecessors' published words (each either a tile's own
+// count or, once that tile has looked back itself, the count of everything up
+// to it) and publishes its inclusive count.  Against a histogram kernel, a scan
+// kernel and a scatter kernel per pass this reads the keys once per pass instead
+// of twice and needs one launch instead of three.
+//
+// Tiles are numbered by a ticket, so a tile's predecessors are always running
+// or done and the wait ends; it is bounded all the same (SPIN_MAX), and a
+// tile that gave up sets GCC_DEVERR_WAIT_BUDGET and stays in bounds.
+template <class W> struct Count {
+    static constexpr int BITS = sizeof(W) * 8 - 2;
+    static constexpr W OWN = W(1) << BITS, UP_TO = W(2) << BITS, MASK = (W(1) << BITS) - 1;
+};
+constexpr uint32_t SPIN_MAX = 1u << 21;
+
+__device__ __forceinline__ uint32_t ld_word(const uint32_t* p) { return ld_relaxed_u32(p); }
+__device__ __forceinline__ uint64_t ld_word(const uint64_t* p) { return ld_relaxed(p); }
+__device__ __forceinline__ void st_word(uint32_t* p, uint32_t v) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_word(uint64_t* p, uint64_t v) { st_relaxed(p, v); }
+
+// Items of digit t (this thread's) in the tiles before `tile`.  Four
+// predecessors are read at once: in the first wave every tile of the grid
+// looks back through unfinished ones, and the reads' latency is what it costs.
+template <class W>
+__device__ __forceinline__ W look_back(const W* desc, int64_t tile, int t, unsigned* err) {
+    constexpr int AHEAD = 4;
+    W sum = 0;
+    uint32_t spins = 0;
+    int64_t p = tile - 1;
+    while (p >= 0) {
+        W w[AHEAD];
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j)
+            w[j] = p - j >= 0 ? ld_word(desc + (p - j) * 256 + t) : Count<W>::UP_TO;
+        int used = 0;
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j) {
+            if (used != j || w[j] == 0) continue;          // not published yet: look again
+            sum += w[j] & Count<W>::MASK;
+            used = w[j] >= Count<W>::UP_TO ? AHEAD + 1 : j + 1;
+        }
+        if (used > AHEAD) break;
+        p -= used;
+        if (used == 0 && ++spins > SPIN_MAX) {
+            if (err) atomicOr(err, GCC_DEVERR_WAIT_BUDGET);
+            break;
+        }
     }
-    __syncthreads();
-    hist[(size_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+    return sum;
 }
 
-// One block per digit: exclusive scan of that digit's per-tile counts.
-__global__ void rs_scan_rows(uint32_t* __restrict__ hist, uint32_t ntiles,
-                             uint32_t* __restrict__ totals) {
-    __shared__ uint32_t warp_sums[32];
-    uint32_t* row = hist + (size_t)blockIdx.x * ntiles;
-    uint32_t carry = 0;
-    for (uint32_t base = 0; base < ntiles; base += 1024) {
-        const uint32_t i = base + threadIdx.x;
-        const uint32_t v = i < ntiles ? row[i] : 0;
-        uint32_t tot;
-        const uint32_t ex = block_exclusive_scan<32>(v, warp_sums, &tot);
-        if (i < ntiles) row[i] = carry + ex;
-        carry += tot;
-    }
-    if (threadIdx.x == 0) totals[blockIdx.x] = carry;
-}
-
-// Stable scatter of one tile.  Each warp ranks its own contiguous run of
-// RS_CHUNKS * 32 items with warp-private digit counters (match_any groups the
-// lanes of one digit; no block barrier inside the loop); one digit-major
-// scan over (digit, warp) then gives every item its position in the tile
-// staged in digit order -- warp w's items of a digit follow warp w-1's, which
-// keeps the sort stable -- and each digit's run goes to its global position
-// with consecutive threads on consecutive addresses (coalesced).
+// Histograms of every pass's digits.
 __global__ void __launch_bounds__(RS_BLOCK)
-rs_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-           uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, size_t n, int shift,
-           const uint32_t* __restrict__ hist, const uint32_t* __restrict__ totals,
-           uint32_t ntiles) {
-    __shared__ uint32_t gbase[256];            // global start of each digit's run for this tile
-    __shared__ uint32_t dstart[256];           // start of each digit within the staged tile
-    __shared__ uint32_t wc[RS_WARPS][256];     // per-warp digit counts, then per-warp starts
-    __shared__ uint32_t skey[RS_TILE];
-    __shared__ uint32_t sval[RS_TILE];
-    __shared__ uint32_t warp_sums[32];
-    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    gbase[t] = block_exclusive_scan<RS_WARPS>(totals[t], warp_sums, nullptr) +
-               hist[(size_t)t * ntiles + blockIdx.x];
-    for (int w = 0; w < RS_WARPS; ++w) wc[w][t] = 0;
+rs_hist(const uint32_t* __restrict__ keys, size_t n, int bits, int passes, int digit_bits,
+        uint32_t* __restrict__ hist) {
+    __shared__ uint32_t h[SORT_MAX_PASSES][256];
+    after_previous();
+    for (int p = 0; p < SORT_MAX_PASSES; ++p) h[p][threadIdx.x] = 0;
     __syncthreads();
-    const size_t tile0 = (size_t)blockIdx.x * RS_TILE;
-    const size_t base = tile0 + (size_t)warp * (RS_CHUNKS * 32);
-    uint32_t key[RS_CHUNKS], val[RS_CHUNKS], rank[RS_CHUNKS];
+    const size_t stride = (size_t)gridDim.x * RS_BLOCK * 4;
+    for (size_t i = ((size_t)blockIdx.x * RS_BLOCK + threadIdx.x) * 4; i < n; i += stride) {
+        uint32_t k[4];
+        const int m = n - i < 4 ? (int)(n - i) : 4;
+        if (m == 4) {
+            const uint4 v = *reinterpret_cast<const uint4*>(keys + i);
+            k[0] = v.x; k[1] = v.y; k[2] = v.z; k[3] = v.w;
+        } else {
+            for (int j = 0; j < m; ++j) k[j] = keys[i + j];
+        }
+        for (int p = 0; p < passes; ++p) {
+            const int left = bits - p * digit_bits;
+            const uint32_t mask = (1u << (left < digit_bits ? left : digit_bits)) - 1u;
 #pragma unroll
-    for (int c = 0; c < RS_CHUNKS; ++c) {
-        const size_t i = base + (size_t)c * 32 + lane;
-        const bool valid = i < n;
-        key[c] = valid ? kin[i] : 0u;
-        val[c] = valid ? vin[i] : 0u;
+            for (int j = 0; j < 4; ++j)
+                if (j < m) atomicAdd(&h[p][(k[j] >> (p * digit_bits)) & mask], 1u);
+        }
     }
+    __syncthreads();
+    for (int p = 0; p < passes; ++p)
+        if (const uint32_t c = h[p][threadIdx.x]) atomicAdd(&hist[p * 256 + threadIdx.x], c);
+}
+
+// One pass over one tile.  Each warp ranks its own contiguous run of ITEMS * 32
+// items with warp-private digit counters: the lanes that share a digit are
+// found with one ballot per digit bit, no block barrier inside the loop.  One
+// digit-major scan over (digit, warp) then gives every item its position in the
+// tile staged in digit order -- warp w's items of a digit follow warp w-1's,
+// which keeps the sort stable -- and each digit's run goes to its global
+// position with consecutive threads on consecutive addresses (coalesced).
+// Bound by issue and by the latency of the ranking's shared-memory round trips,
+// not by memory (2^24 pairs: 0.14 ms a pass, 1.9 TB/s).  16 items per thread
+// took 1.52 ms for a 2^24-op deterministic batch, 8 items 1.61 ms, 12 items
+// 1.60 ms; __match_any_sync instead of the ballots 1.69 ms; a minimum of 3 or
+// 4 resident blocks (spills) and loading the values behind the ranking were
+// slower too.
+// `flagged` (first pass of radix_sort_positions): values are positions, bit 31
+// of the key moves to bit 31 of the value.
+template <class W, int ITEMS>
+__global__ void __launch_bounds__(RS_BLOCK)
+rs_pass(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
+        uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, size_t n, int shift, int width,
+        int flagged, const uint32_t* __restrict__ hist, W* desc, W* desc_next, uint32_t* ticket,
+        unsigned* err) {
+    constexpr int TILE = RS_BLOCK * ITEMS;
+    __shared__ uint32_t gbase[256];            // global start of each digit's run, less dstart
+    __shared__ uint32_t wc[RS_WARPS][256];     // per-warp digit counts, then starts in the tile
+    __shared__ uint32_t skey[TILE];
+    __shared__ uint32_t sval[TILE];
+    __shared__ uint32_t warp_sums[32];
+    __shared__ uint32_t s_tile;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
 #pragma unroll
-    for (int c = 0; c < RS_CHUNKS; ++c) {
-        const bool valid = base + (size_t)c * 32 + lane < n;
-        const uint32_t dg = valid ? (key[c] >> shift) & 255u : 256u;
-        const unsigned peers = __match_any_sync(0xffffffffu, dg);
+    for (int w = 0; w < RS_WARPS; ++w) wc[w][t] = 0;
+    after_previous();
+    if (t == 0) s_tile = atomicAdd(ticket, 1u);
+    __syncthreads();
+    const uint32_t tile = s_tile;
+    const size_t tile0 = (size_t)tile * TILE;
+    const uint32_t tile_n = (uint32_t)(n - tile0 < (size_t)TILE ? n - tile0 : (size_t)TILE);
+    const uint32_t base = (uint32_t)warp * (ITEMS * 32) + lane;    // the thread's first item of the tile
+    kin += tile0;
+    const uint32_t dmask = (1u << width) - 1u;
+    uint32_t key[ITEMS], val[ITEMS];
+    uint16_t rank[ITEMS];
+#pragma unroll
+    for (int c = 0; c < ITEMS; ++c) key[c] = base + c * 32 < tile_n ? kin[base + c * 32] : 0u;
+    if (vin) {
+        vin += tile0;
+#pragma unroll
+        for (int c = 0; c < ITEMS; ++c) val[c] = base + c * 32 < tile_n ? vin[base + c * 32] : 0u;
+    } else {
+#pragma unroll
+        for (int c = 0; c < ITEMS; ++c) {
+            val[c] = (uint32_t)tile0 + base + c * 32;
+            if (flagged) {
+                val[c] |= key[c] & 0x80000000u;
+                key[c] &= 0x7fffffffu;
+            }
+        }
+    }
+    desc_next[(size_t)tile * 256 + t] = 0;     // the next pass's descriptors start unpublished
+    const uint32_t in_hist = hist[t];
+#pragma unroll
+    for (int c = 0; c < ITEMS; ++c) {
+        const bool valid = base + c * 32 < tile_n;
+        const uint32_t dg = (key[c] >> shift) & dmask;
+        unsigned peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {          // bits from `width` on are zero in every lane
+            const int x = (int)(dg << (31 - b)) >> 31;
+            const unsigned m = __ballot_sync(0xffffffffu, x);
+            peers &= ~(m ^ (unsigned)x);
+        }
         const uint32_t prior = valid ? wc[warp][dg] : 0u;
         __syncwarp();
         if (valid && (peers & lt_mask()) == 0) wc[warp][dg] = prior + __popc(peers);
         __syncwarp();
-        rank[c] = prior + __popc(peers & lt_mask());
+        rank[c] = (uint16_t)(prior + __popc(peers & lt_mask()));
     }
     __syncthreads();
-    uint32_t tot = 0;                          // thread t owns digit t
+    uint32_t cnt[RS_WARPS], tot = 0;           // thread t owns digit t
+#pragma unroll
     for (int w = 0; w < RS_WARPS; ++w) {
-        const uint32_t x = wc[w][t];
-        wc[w][t] = tot;
-        tot += x;
+        cnt[w] = tot;
+        tot += wc[w][t];
     }
-    dstart[t] = block_exclusive_scan<RS_WARPS>(tot, warp_sums, nullptr);
+    st_word(desc + (size_t)tile * 256 + t, (tile ? Count<W>::OWN : Count<W>::UP_TO) | (W)tot);
+    const uint32_t dstart = block_exclusive_scan<RS_WARPS>(tot, warp_sums, nullptr);
+    const uint32_t gstart = block_exclusive_scan<RS_WARPS>(in_hist, warp_sums, nullptr);
+#pragma unroll
+    for (int w = 0; w < RS_WARPS; ++w) wc[w][t] = dstart + cnt[w];
     __syncthreads();
 #pragma unroll
-    for (int c = 0; c < RS_CHUNKS; ++c) {
-        if (base + (size_t)c * 32 + lane < n) {
-            const uint32_t dg = (key[c] >> shift) & 255u;
-            const uint32_t pos = dstart[dg] + wc[warp][dg] + rank[c];
+    for (int c = 0; c < ITEMS; ++c) {
+        if (base + c * 32 < tile_n) {
+            const uint32_t pos = wc[warp][(key[c] >> shift) & dmask] + rank[c];
             skey[pos] = key[c];
             sval[pos] = val[c];
         }
     }
-    __syncthreads();
-    const uint32_t tile_n = (uint32_t)((n - tile0) < (size_t)RS_TILE ? (n - tile0) : RS_TILE);
-    for (uint32_t i = t; i < tile_n; i += RS_BLOCK) {
-        const uint32_t k = skey[i];
-        const uint32_t dg = (k >> shift) & 255u;
-        const uint32_t out = gbase[dg] + (i - dstart[dg]);
-        kout[out] = k;
-        vout[out] = sval[i];
+    if (tile) {
+        const W before = look_back<W>(desc, tile, t, err);
+        st_word(desc + (size_t)tile * 256 + t, Count<W>::UP_TO | (before + (W)tot));
+        gbase[t] = gstart + (uint32_t)before - dstart;
+    } else {
+        gbase[t] = gstart - dstart;
     }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < ITEMS; ++c) {
+        const uint32_t i = (uint32_t)c * RS_BLOCK + t;
+        if (i < tile_n) {
+            const uint32_t k = skey[i];
+            const uint32_t out = gbase[(k >> shift) & dmask] + i;
+            if (out < n) {                     // a bounded wait that gave up stays in bounds
+                kout[out] = k;
+                vout[out] = sval[i];
+            }
+        }
+    }
+}
+
+template <class W, int ITEMS>
+cudaError_t rs_passes(SortScratch& s, uint32_t* keys, uint32_t* vals, size_t n, int bits, bool flagged,
+                      uint32_t** keys_out, uint32_t** vals_out, cudaStream_t st) {
+    const SortPlan plan = sort_plan(bits);
+    const unsigned tiles = (unsigned)sort_tiles(n);
+    uint32_t *ki = keys, *vi = vals, *ko = s.k1, *vo = s.v1;
+    W* desc = reinterpret_cast<W*>(s.work + SORT_DESC);
+    W* next = desc + (size_t)tiles * 256;
+    for (int p = 0; p < plan.passes; ++p) {
+        const cudaError_t e = launch_after(
+            rs_pass<W, ITEMS>, tiles, RS_BLOCK, st, ki, vi, ko, vo, n, p * plan.digit_bits,
+            plan.width(bits, p), flagged && p == 0 ? 1 : 0, s.work + SORT_HIST + p * 256, desc, next,
+            s.work + p, s.err);
+        if (e != cudaSuccess) return e;
+        uint32_t* tk = ki; ki = ko; ko = tk;
+        uint32_t* tv = vi ? vi : s.v0; vi = vo; vo = tv;
+        W* td = desc; desc = next; next = td;
+    }
+    *keys_out = ki;
+    *vals_out = vi;
+    return cudaSuccess;
+}
+
+cudaError_t rs_run(SortScratch& s, uint32_t* keys, uint32_t* vals, size_t n, int bits, bool flagged,
+                   uint32_t** keys_out, uint32_t** vals_out, cudaStream_t st) {
+    if (n <= SORT_SMALL)
+        return rs_passes<uint32_t, SORT_ITEMS_SMALL>(s, keys, vals, n, bits, flagged, keys_out, vals_out, st);
+    if (n < (size_t(1) << 30))
+        return rs_passes<uint32_t, SORT_ITEMS_LARGE>(s, keys, vals, n, bits, flagged, keys_out, vals_out, st);
+    return rs_passes<uint64_t, SORT_ITEMS_LARGE>(s, keys, vals, n, bits, flagged, keys_out, vals_out, st);
 }
 
 // --- prefix sum -------------------------------------------------------------
@@ -318,23 +450,34 @@ inline unsigned blocks_for(uint64_t n, int b) { return (unsigned)((n + b - 1) / 
 
 }  // namespace
 
-size_t sort_max_tiles(size_t n) { return (n + RS_TILE - 1) / RS_TILE; }
+// Zeroed tickets and descriptors, and the histograms of every pass.
+static cudaError_t rs_prepare(SortScratch& s, const uint32_t* keys, size_t n, int bits, cudaStream_t st) {
+    const SortPlan plan = sort_plan(bits);
+    const cudaError_t e = cudaMemsetAsync(s.work, 0, (SORT_DESC + sort_desc_words(n)) * 4, st);
+    if (e != cudaSuccess) return e;
+    const unsigned grid = blocks_for(n, RS_BLOCK * 4 * 4);
+    return launch_after(rs_hist, grid < 608u ? grid : 608u, RS_BLOCK, st, keys, n, bits, plan.passes,
+                        plan.digit_bits, s.work + SORT_HIST);
+}
 
 cudaError_t radix_sort_pairs(SortScratch& s, size_t n, int bits, uint32_t** keys_out,
                              uint32_t** vals_out, cudaStream_t st) {
-    uint32_t *ki = s.k0, *vi = s.v0, *ko = s.k1, *vo = s.v1;
-    if (n == 0) { *keys_out = ki; *vals_out = vi; return cudaSuccess; }
-    const uint32_t ntiles = (uint32_t)sort_max_tiles(n);
-    for (int shift = 0; shift < bits; shift += 8) {
-        rs_hist<<<ntiles, RS_BLOCK, 0, st>>>(ki, n, shift, s.hist, ntiles);
-        rs_scan_rows<<<256, 1024, 0, st>>>(s.hist, ntiles, s.totals);
-        rs_scatter<<<ntiles, RS_BLOCK, 0, st>>>(ki, vi, ko, vo, n, shift, s.hist, s.totals, ntiles);
-        uint32_t* tk = ki; ki = ko; ko = tk;
-        uint32_t* tv = vi; vi = vo; vo = tv;
+    if (n == 0) { *keys_out = s.k0; *vals_out = s.v0; return cudaSuccess; }
+    const cudaError_t e = rs_prepare(s, s.k0, n, bits, st);
+    if (e != cudaSuccess) return e;
+    return rs_run(s, s.k0, s.v0, n, bits, false, keys_out, vals_out, st);
+}
+
+int radix_sort_launches(int bits) { return 1 + sort_plan(bits).passes; }
+
+cudaError_t radix_sort_positions(SortScratch& s, uint32_t* keys, size_t n, int bits, bool flagged,
+                                 bool prepared, uint32_t** keys_out, uint32_t** vals_out,
+                                 cudaStream_t st) {
+    if (!prepared) {
+        const cudaError_t e = rs_prepare(s, keys, n, bits, st);
+        if (e != cudaSuccess) return e;
     }
-    *keys_out = ki;
-    *vals_out = vi;
-    return cudaGetLastError();
+    return rs_run(s, keys, nullptr, n, bits, flagged, keys_out, vals_out, st);
 }
 
 size_t scan_tmp_words(size_t n) { return (n + SC_TILE - 1) / SC_TILE + 1; }
