@@ -194,8 +194,7 @@ typedef struct gcc_exec_params {
                                   no delay (the paper's policy) [0] */
     uint32_t det_dataflow;     /* GCC_DET: 0 = evaluate each record's chain in one
                                   pass over the batch's accesses sorted by record
-                                  (key-value: prefix sums; order-entry: one warp
-                                  per record applies its ops in id order)
+                                  (prefix sums along each record's accesses)
                                   [default; key-value needs n_records *
                                   n_fields below 2^32, else the batch is
                                   refused with GCC_ERR_CAPACITY]; 1 = run op

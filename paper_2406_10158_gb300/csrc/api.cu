@@ -153,6 +153,7 @@ void free_db(gcc_db* db) {
     cudaFree(db->unit_link);
     cudaFree(db->name_idx);
     cudaFree(db->name_last);
+    cudaFree(db->name_pick);
     cudaFree(db->ops_resolved);
     if (db->h_states) cudaFreeHost(db->h_states);
     for (auto& r : db->stages)
@@ -220,10 +221,11 @@ gcc_status create_impl(const gcc_db_desc* desc, gcc_db** out) {
         const uint64_t n_cust = W * OE_DIST * OE_CUST;
         if ((s = dev_alloc(&db->name_idx, n_cust * 4, "last-name index"))) return bail(s);
         if ((s = dev_alloc(&db->name_last, n_cust * 8, "last-name index"))) return bail(s);
+        if ((s = dev_alloc(&db->name_pick, W * OE_DIST * gcc::NAME_PICKS * 4, "last-name index"))) return bail(s);
         if ((s = dev_alloc(&db->ops_resolved, d.max_batch_ops * 8, "resolved ops"))) return bail(s);
         if (gcc::build_name_index(db->cols[gcc::rt::OE_C_LAST], db->cols[gcc::rt::OE_C_FIRST],
                                   (uint32_t)(W * OE_DIST), db->name_idx, db->name_last,
-                                  db->stream) != cudaSuccess ||
+                                  db->name_pick, db->stream) != cudaSuccess ||
             cudaStreamSynchronize(db->stream) != cudaSuccess)
             return bail(fail(GCC_ERR_CUDA, "cannot build the last-name index"));
     }
@@ -245,8 +247,10 @@ gcc_status create_impl(const gcc_db_desc* desc, gcc_db** out) {
     if ((s = dev_alloc(&db->order_key, d.max_batch_txns * 8, "commit keys"))) return bail(s);
     if ((s = dev_alloc(&db->fold_flags, d.max_batch_txns * 8, "validity flags and ranks")))
         return bail(s);
-    if (d.schema == GCC_SCHEMA_KV &&
-        (s = dev_alloc(&db->fold_seg, gcc::fold_seg_bytes(d.max_batch_ops, d.max_batch_txns),
+    if ((s = dev_alloc(reinterpret_cast<uint8_t**>(&db->fold_seg),
+                       d.schema == GCC_SCHEMA_KV
+                           ? gcc::fold_seg_bytes(d.max_batch_ops, d.max_batch_txns)
+                           : gcc::oe_scratch_bytes(d.max_batch_ops, d.max_batch_txns),
                        "fold descriptors")))
         return bail(s);
     // MVCC version pointers, one per slot, zero between batches
@@ -383,45 +387,32 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
     a.queue_after = queue_after_for(p, scheme);
 
     const bool kv = db->d.schema == GCC_SCHEMA_KV;
-    // deterministic key-value batches: every record chain by prefix sums (the
-    // pipeline begins the batch itself)
-    const bool fold = scheme == GCC_DET && kv && !p.det_dataflow;
+    // deterministic batches: every record chain by prefix sums (the pipelines
+    // begin the batch themselves)
+    const bool fold = scheme == GCC_DET && !p.det_dataflow;
     if (!fold) {
         GCC_CK(gcc::launch_batch_begin(db->st, db->dbs, scheme, st));
         launches += 1;
     }
-    if (!kv && n_ops) {
+    if (!kv && n_ops && !fold) {
         // payments by last name become payments of the customer they name,
         // before any scheme sees the batch
-        GCC_CK(gcc::resolve_by_name(a.ops, n_ops, db->d.n_warehouses, db->name_idx, db->name_last,
+        GCC_CK(gcc::resolve_by_name(a.ops, n_ops, db->d.n_warehouses,
+                                    gcc::NameIndex{db->name_idx, db->name_last, db->name_pick},
                                     db->ops_resolved, st));
         a.ops = db->ops_resolved;
         launches += 1;
     }
     if (fold) {
         GCC_CK(cudaEventRecord(rec.ev[1], st));
-        GCC_CK(gcc::det_fold_kv(a, db->d.field_bytes, db->sort, db->fold_seg, launches, st));
-        GCC_CK(cudaEventRecord(rec.ev[2], st));
-        GCC_CK(cudaEventRecord(rec.ev[3], st));
-        rec.stream = st;
-        rec.scheme = scheme;
-        rec.n_txns = n_txns;
-        rec.launches = launches;
-        rec.grid = 0;
-        rec.used = true;
-        db->n_stages++;                  // control words untouched
-        db->last_stream = st;
-        db->last_scheme = scheme;
-        db->last_n_txns = n_txns;
-        return GCC_OK;
-    }
-    // deterministic order-entry batches: every record chain in one pass
-    if (scheme == GCC_DET && !kv && !p.det_dataflow) {
-        const int bits = std::max(1, bit_length(db->n_meta));
-        GCC_CK(cudaEventRecord(rec.ev[1], st));
-        GCC_CK(gcc::det_serial_oe(a, db->sort, db->scan_tmp, db->fold_flags, db->need, bits,
-                                  db->sm_count, st));
-        launches += gcc::det_serial_oe_launches(bits);
+        if (kv) {
+            GCC_CK(gcc::det_fold_kv(a, db->d.field_bytes, db->sort, db->fold_seg, launches, st));
+        } else {
+            gcc::OeTables T{};
+            for (int c = 0; c < OE_NCOLS; ++c) T.c[c] = reinterpret_cast<uint64_t*>(db->cols[c]);
+            T.names = gcc::NameIndex{db->name_idx, db->name_last, db->name_pick};
+            GCC_CK(gcc::det_serial_oe(a, T, db->sort, db->fold_seg, db->need, launches, st));
+        }
         GCC_CK(cudaEventRecord(rec.ev[2], st));
         GCC_CK(cudaEventRecord(rec.ev[3], st));
         rec.stream = st;
@@ -618,7 +609,7 @@ gcc_status gcc_load_table(gcc_db* db, uint32_t id, const void* src, uint64_t nby
         (id == (uint32_t)gcc::rt::OE_C_LAST || id == (uint32_t)gcc::rt::OE_C_FIRST))
         GCC_CK(gcc::build_name_index(db->cols[gcc::rt::OE_C_LAST], db->cols[gcc::rt::OE_C_FIRST],
                                      db->d.n_warehouses * gcc::rt::OE_DIST, db->name_idx,
-                                     db->name_last, nullptr));
+                                     db->name_last, db->name_pick, nullptr));
     GCC_CK(cudaDeviceSynchronize());
     return GCC_OK;
 }

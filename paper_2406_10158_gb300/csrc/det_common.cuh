@@ -19,6 +19,70 @@ constexpr uint32_t DET_SPIN_MAX = 1u << 21;
 
 inline unsigned blocks_for(uint64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
+// The sort keys of a batch's accesses: bits 0..rec_bits-1 the record or slot
+// (`none`: the op takes no part), above it the op's chunk, bit 31 (`flagged`)
+// one bit of the caller's that the sort hands on in the value.
+struct AccessKeys {
+    uint32_t none;
+    int rec_bits, bits, passes, digit_bits, chunk_log2, sort_log2;
+    int flagged;
+    __device__ uint32_t key(uint64_t op, uint32_t rec, bool flag) const {
+        uint32_t k = rec;
+        if (bits > rec_bits) k |= ((uint32_t)(op & ((1ull << sort_log2) - 1)) >> chunk_log2) << rec_bits;
+        return k | (flagged && flag ? 0x80000000u : 0u);
+    }
+    __device__ uint32_t rec(uint32_t k) const { return rec_bits == 32 ? k : k & ((1u << rec_bits) - 1u); }
+    // the op of a sorted value, positions counting from op0
+    __device__ uint64_t op(uint64_t op0, uint32_t v) const { return op0 + (flagged ? v & 0x7fffffffu : v); }
+};
+
+inline AccessKeys access_keys(uint64_t none, uint64_t n_ops, int chunk_log2, int sort_log2, bool flag) {
+    AccessKeys f;
+    f.none = (uint32_t)none;
+    f.rec_bits = 0;
+    for (uint64_t v = none; v; v >>= 1) ++f.rec_bits;
+    const uint64_t m = std::min<uint64_t>(n_ops, 1ull << sort_log2);
+    int want = 0;                            // chunk bits
+    while (((uint64_t)1 << (chunk_log2 + want)) < m) ++want;
+    f.flagged = flag && f.rec_bits <= 31;
+    const int chunk_bits = std::min(want, (f.flagged ? 31 : 32) - f.rec_bits);
+    f.chunk_log2 = chunk_log2 + (want - chunk_bits);
+    f.sort_log2 = sort_log2;
+    f.bits = f.rec_bits + chunk_bits;
+    const SortPlan sp = sort_plan(f.bits);
+    f.passes = sp.passes;
+    f.digit_bits = sp.digit_bits;
+    return f;
+}
+
+// Scratch of a pass, zeroed by det_begin: a ticket and a list length per chunk,
+// one word per tile of transactions (det_finish), one descriptor per tile of ops.
+struct DetScratch {
+    uint32_t *tickets, *lengths;
+    unsigned long long* rank_desc;
+    ulonglong2* tile_desc;
+    ulonglong2* zero;
+    size_t n_zero;
+};
+constexpr uint32_t RANK_TILE = 1024;
+inline DetScratch det_scratch(void* base, uint64_t n_ops, uint64_t n_txns, int chunk_log2, int tile) {
+    const auto rounded = [](size_t b) { return (b + 255) & ~size_t(255); };
+    char* p = static_cast<char*>(base);
+    DetScratch s;
+    s.zero = reinterpret_cast<ulonglong2*>(p);
+    const size_t chunks = rounded(((size_t)(n_ops >> chunk_log2) + 2) * 4);
+    s.tickets = reinterpret_cast<uint32_t*>(p);
+    p += chunks;
+    s.lengths = reinterpret_cast<uint32_t*>(p);
+    p += chunks;
+    s.rank_desc = reinterpret_cast<unsigned long long*>(p);
+    p += rounded((n_txns / RANK_TILE + 1) * 8);
+    s.tile_desc = reinterpret_cast<ulonglong2*>(p);
+    p += rounded((n_ops / tile + 2) * 16);
+    s.n_zero = (size_t)(p - static_cast<char*>(base)) / 16;
+    return s;
+}
+
 // A block-wide election: true in every thread of the last block to arrive at
 // `counter` (which is left at zero), whose accesses then follow every other
 // block's.
@@ -40,12 +104,11 @@ __device__ __forceinline__ bool last_block(uint32_t* counter) {
 // but the words above) and the pass's own descriptors (`zero2`), and checks that
 // the transactions' op ranges tile ops[0, n_ops) in id order, which the
 // contract asks for.  Where they do not, DW_UNTILED is set and the last block
-// gives every op the key `none(i)`, so that an op outside every range stays out
-// of the access table; the validation pass then overwrites the others'.
-template <class None>
+// gives every op the key of no record, so that an op outside every range stays
+// out of the access table; the validation pass then overwrites the others'.
 __global__ void __launch_bounds__(256)
 det_begin(const __grid_constant__ ExecArgs a, uint32_t* work, ulonglong2* zero, size_t n_zero,
-          ulonglong2* zero2, size_t n_zero2, uint32_t* keys, None none) {
+          ulonglong2* zero2, size_t n_zero2, uint32_t* keys, const AccessKeys f) {
     after_previous();
     const size_t i0 = (size_t)blockIdx.x * 256 + threadIdx.x, stride = (size_t)gridDim.x * 256;
     if (i0 == 0) {
@@ -78,7 +141,19 @@ det_begin(const __grid_constant__ ExecArgs a, uint32_t* work, ulonglong2* zero, 
         work[DW_UNTILED_ACC] = 0;
     }
     if (bad)
-        for (uint64_t i = threadIdx.x; i < a.n_ops; i += 256) keys[i] = none(i);
+        for (uint64_t i = threadIdx.x; i < a.n_ops; i += 256) keys[i] = f.key(i, f.none, false);
+}
+
+// Launches det_begin; with one sort for the whole batch (`one_sort`) it also
+// prepares that sort's tickets, histograms and descriptors.
+inline cudaError_t launch_det_begin(const ExecArgs& a, SortScratch& s, const DetScratch& sc,
+                                    const AccessKeys& f, bool one_sort, cudaStream_t st) {
+    const size_t n_zero = one_sort ? (SORT_DESC - SORT_HIST + sort_desc_words(a.n_ops)) / 4 : 0;
+    const uint64_t most = std::max<uint64_t>(std::max<uint64_t>(n_zero, sc.n_zero), a.n_txns);
+    const unsigned grid = std::min<unsigned>(std::max<unsigned>(blocks_for(most, 256), 1u), 608u);
+    return launch_after(det_begin, grid, 256, st, a, s.work,
+                        reinterpret_cast<ulonglong2*>(s.work + SORT_HIST), n_zero, sc.zero, sc.n_zero,
+                        s.k0, f);
 }
 
 // The block's digit histograms: HIST_COPIES copies side by side, a lane adding
@@ -86,14 +161,15 @@ det_begin(const __grid_constant__ ExecArgs a, uint32_t* work, ulonglong2* zero, 
 // (the top digits of neighbouring ops often are) rarely meet on one word.
 constexpr int HIST_COPIES = 4;
 typedef uint32_t DigitHist[256 * HIST_COPIES];
-__device__ __forceinline__ void count_digits(DigitHist* h, uint32_t k, int bits, int passes, int digit_bits) {
+__device__ __forceinline__ void count_digits(DigitHist* h, uint32_t k, int bits, int passes, int digit_bits,
+                                             uint32_t times = 1u) {
     const uint32_t copy = threadIdx.x % HIST_COPIES;
 #pragma unroll
     for (int p = 0; p < SORT_MAX_PASSES; ++p)
         if (p < passes) {
             const int left = bits - p * digit_bits;
             const uint32_t mask = (1u << (left < digit_bits ? left : digit_bits)) - 1u;
-            atomicAdd(&h[p][((k >> (p * digit_bits)) & mask) * HIST_COPIES + copy], 1u);
+            atomicAdd(&h[p][((k >> (p * digit_bits)) & mask) * HIST_COPIES + copy], times);
         }
 }
 __device__ __forceinline__ void clear_digits(DigitHist* h) {
@@ -130,7 +206,6 @@ __device__ __forceinline__ void flush_digits(DigitHist* h, uint32_t* work, const
 // transaction is valid; otherwise the order is the rank among the valid ones,
 // by one scan over tiles of transactions with look-back (rank_desc: one zeroed
 // word per tile of 1024).
-constexpr uint32_t RANK_TILE = 1024;
 __global__ void __launch_bounds__(1024)
 det_finish(const __grid_constant__ ExecArgs a, uint32_t* work, unsigned long long* rank_desc) {
     __shared__ uint32_t s_tile, s_warp[32], s_before;
@@ -193,6 +268,11 @@ det_finish(const __grid_constant__ ExecArgs a, uint32_t* work, unsigned long lon
         __syncthreads();
         if (ok) a.results[t].commit_order = s_before + s_warp[warp] + __popc(m & lanemask_lt());
     }
+}
+
+inline cudaError_t launch_det_finish(const ExecArgs& a, SortScratch& s, const DetScratch& sc, cudaStream_t st) {
+    return launch_after(det_finish, std::min<unsigned>(blocks_for(a.n_txns, RANK_TILE), 152u), 1024, st, a,
+                        s.work, sc.rank_desc);
 }
 
 }  // namespace

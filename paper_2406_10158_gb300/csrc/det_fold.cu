@@ -51,77 +51,12 @@ __device__ __forceinline__ uint32_t d_key(uint64_t d) { return (uint32_t)d; }
 __device__ __forceinline__ uint32_t d_field(uint64_t d) { return (uint32_t)(d >> 32) & 0xffu; }
 __device__ __forceinline__ uint32_t d_kind(uint64_t d) { return (uint32_t)(d >> 40) & 0xffu; }
 
-// The sort keys of a batch: bits 0..slot_bits-1 the slot (n_slots: none),
-// above it the op's chunk, bit 31 (when free) whether the op is an ADD.
-struct FoldKeys {
-    uint32_t n_slots;
-    int slot_bits, bits, passes, digit_bits, chunk_log2;
-    int flagged;
-    __host__ __device__ uint32_t chunk_of(uint64_t op) const {
-        return (uint32_t)(op & ((1ull << SORT_LOG2) - 1)) >> chunk_log2;
-    }
-    __device__ uint32_t key(uint64_t op, uint32_t slot, bool add) const {
-        uint32_t k = slot | (bits > slot_bits ? chunk_of(op) << slot_bits : 0u);
-        return k | (flagged && add ? 0x80000000u : 0u);
-    }
-    __device__ uint32_t slot(uint32_t k) const {
-        return slot_bits == 32 ? k : k & ((1u << slot_bits) - 1u);
-    }
-    // the op of a sorted value, positions counting from op0
-    __device__ uint64_t op(uint64_t op0, uint32_t v) const { return op0 + (flagged ? v & 0x7fffffffu : v); }
-    __device__ uint32_t operator()(uint64_t op) const { return key(op, n_slots, false); }
-};
-
-FoldKeys fold_keys(uint64_t n_slots, uint64_t n_ops) {
-    FoldKeys f;
-    f.n_slots = (uint32_t)n_slots;
-    f.slot_bits = 0;
-    for (uint64_t v = n_slots; v; v >>= 1) ++f.slot_bits;
-    const uint64_t m = std::min<uint64_t>(n_ops, 1ull << SORT_LOG2);
-    int want = 0;                            // chunk bits
-    while (((uint64_t)1 << (CHUNK_LOG2 + want)) < m) ++want;
-    f.flagged = f.slot_bits <= 31;
-    const int room = f.flagged ? 31 - f.slot_bits : 0;
-    const int chunk_bits = std::min(want, room);
-    f.chunk_log2 = CHUNK_LOG2 + (want - chunk_bits);
-    f.bits = f.slot_bits + chunk_bits;
-    const SortPlan sp = sort_plan(f.bits);
-    f.passes = sp.passes;
-    f.digit_bits = sp.digit_bits;
-    return f;
-}
-
 // A running sum in the slot's lane arithmetic.
 struct Sum {
     uint64_t lo;
     uint32_t hi;           // modulo 2^16
 };
 __device__ __forceinline__ Sum sum_add(Sum a, Sum b) { return Sum{a.lo + b.lo, (a.hi + b.hi) & 0xFFFFu}; }
-
-// Scratch (zeroed by det_begin): one ticket per chunk, one word per tile of
-// transactions (det_finish), one descriptor per tile of ops.
-struct FoldScratch {
-    uint32_t* tickets;
-    unsigned long long* rank_desc;
-    ulonglong2* tile_desc;
-    ulonglong2* zero;
-    size_t n_zero;
-};
-size_t rounded(size_t bytes) { return (bytes + 255) & ~size_t(255); }
-size_t chunks_of(uint64_t n_ops) { return (size_t)(n_ops >> CHUNK_LOG2) + 2; }
-FoldScratch fold_scratch(void* base, uint64_t n_ops, uint64_t n_txns) {
-    char* p = static_cast<char*>(base);
-    FoldScratch s;
-    s.zero = reinterpret_cast<ulonglong2*>(p);
-    s.tickets = reinterpret_cast<uint32_t*>(p);
-    p += rounded(chunks_of(n_ops) * 4);
-    s.rank_desc = reinterpret_cast<unsigned long long*>(p);
-    p += rounded((n_txns / RANK_TILE + 1) * 8);
-    s.tile_desc = reinterpret_cast<ulonglong2*>(p);
-    p += rounded((n_ops / FT_TILE<16> + 2) * 16);
-    s.n_zero = (size_t)(p - static_cast<char*>(base)) / 16;
-    return s;
-}
 
 // --- validation and access table ---------------------------------------------
 // A lane group of G lanes per transaction (G the smallest of 8, 16, 32 that
@@ -132,7 +67,7 @@ FoldScratch fold_scratch(void* base, uint64_t n_ops, uint64_t n_txns) {
 // updates (one per op and pass).
 template <int G>
 __global__ void __launch_bounds__(256)
-fold_validate(const __grid_constant__ ExecArgs a, const FoldKeys f, uint32_t* __restrict__ keys,
+fold_validate(const __grid_constant__ ExecArgs a, const AccessKeys f, uint32_t* __restrict__ keys,
               uint32_t* work, uint32_t per_block) {
     constexpr int GROUPS = 256 / G, U = G == 32 ? 2 : 4;
     __shared__ DigitHist h[SORT_MAX_PASSES];
@@ -196,7 +131,7 @@ fold_validate(const __grid_constant__ ExecArgs a, const FoldKeys f, uint32_t* __
             const bool no = bad[u] || (any & gmask);
             if (has) {
                 const uint64_t op = (uint64_t)first[u] + lig;
-                const uint32_t k = f.key(op, no ? f.n_slots : d_field(d[u]) * (uint32_t)a.n_records + d_key(d[u]),
+                const uint32_t k = f.key(op, no ? f.none : d_field(d[u]) * (uint32_t)a.n_records + d_key(d[u]),
                                          !no && d_kind(d[u]) == GCC_OP_ADD);
                 keys[op] = k;
                 if (tiled) count_digits(h, k, f.bits, f.passes, f.digit_bits);
@@ -205,7 +140,7 @@ fold_validate(const __grid_constant__ ExecArgs a, const FoldKeys f, uint32_t* __
             if (inside[u] && (bad[u] || nops[u] > G)) {
                 for (uint32_t j = (bad[u] ? 0u : (uint32_t)G) + lig; j < nops[u]; j += G) {
                     const uint64_t op = (uint64_t)first[u] + j;
-                    const uint32_t k = f.key(op, no ? f.n_slots : d_field(d2) * (uint32_t)a.n_records + d_key(d2),
+                    const uint32_t k = f.key(op, no ? f.none : d_field(d2) * (uint32_t)a.n_records + d_key(d2),
                                              !no && d_kind(d2) == GCC_OP_ADD);
                     keys[op] = k;
                     if (tiled) count_digits(h, k, f.bits, f.passes, f.digit_bits);
@@ -294,7 +229,7 @@ __device__ __forceinline__ Sum fold_look_back(const ulonglong2* desc, int64_t ti
 // eight launches of this one 0.83 ms.
 template <int FB>
 __global__ void __launch_bounds__(FT_THREADS, 4)
-fold_tiles(const __grid_constant__ ExecArgs a, const FoldKeys f, const uint32_t* __restrict__ sk,
+fold_tiles(const __grid_constant__ ExecArgs a, const AccessKeys f, const uint32_t* __restrict__ sk,
            const uint32_t* __restrict__ sv, uint64_t op0, uint32_t c0, uint32_t c1,
            uint32_t* ticket, ulonglong2* desc) {
     constexpr int ITEMS = FT_ITEMS<FB>;
@@ -339,12 +274,12 @@ fold_tiles(const __grid_constant__ ExecArgs a, const FoldKeys f, const uint32_t*
     uint32_t seen = 0;
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-        const bool in = base + i < c1 && f.slot(k[i]) < f.n_slots && f.op(op0, v[i]) < a.n_ops;
+        const bool in = base + i < c1 && f.rec(k[i]) < f.none && f.op(op0, v[i]) < a.n_ops;
         live |= in ? 1u << i : 0u;
         if (!in || (i == 0 ? base == c0 || prev != k[0] : k[i - 1] != k[i])) head |= 1u << i;
         dl[i] = Sum{0, 0};
         init[i] = make_ulonglong2(0ull, 0ull);
-        if (in) init[i] = slot_load<FB>(a, f.slot(k[i]));
+        if (in) init[i] = slot_load<FB>(a, f.rec(k[i]));
     }
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i)
@@ -422,7 +357,7 @@ fold_tiles(const __grid_constant__ ExecArgs a, const FoldKeys f, const uint32_t*
         const bool last = base + i + 1 >= c1 || (i + 1 < ITEMS ? k[(i + 1) % ITEMS] : next) != k[i];
         if (last && (carry.lo | carry.hi)) {                     // unchanged slots are not stored
             const ulonglong2 fin = slot_plus<FB>(init[i], carry);
-            uint8_t* dst = a.table + (uint64_t)f.slot(k[i]) * FB;
+            uint8_t* dst = a.table + (uint64_t)f.rec(k[i]) * FB;
             if (FB == 16) *reinterpret_cast<ulonglong2*>(dst) = fin;
             else *reinterpret_cast<uint64_t*>(dst) = fin.x;
         }
@@ -432,15 +367,10 @@ fold_tiles(const __grid_constant__ ExecArgs a, const FoldKeys f, const uint32_t*
 template <int FB>
 cudaError_t fold_run(const ExecArgs& a, SortScratch& s, void* scratch, uint32_t& launches, cudaStream_t st) {
     const uint64_t n = a.n_ops;
-    const FoldKeys f = fold_keys((uint64_t)a.n_fields * a.n_records, n);
-    const FoldScratch sc = fold_scratch(scratch, n, a.n_txns);
+    const AccessKeys f = access_keys((uint64_t)a.n_fields * a.n_records, n, CHUNK_LOG2, SORT_LOG2, true);
+    const DetScratch sc = det_scratch(scratch, n, a.n_txns, CHUNK_LOG2, FT_TILE<16>);
     const bool one_sort = n <= (1ull << SORT_LOG2);
-    const size_t n_zero = one_sort ? (SORT_DESC - SORT_HIST + sort_desc_words(n)) / 4 : 0;
-    const uint64_t most = std::max<uint64_t>(std::max<uint64_t>(n_zero, sc.n_zero), a.n_txns);
-    const unsigned grid0 = std::min<unsigned>(std::max<unsigned>(blocks_for(most, 256), 1u), 608u);
-    cudaError_t e = launch_after(det_begin<FoldKeys>, grid0, 256, st, a, s.work,
-                                 reinterpret_cast<ulonglong2*>(s.work + SORT_HIST), n_zero, sc.zero,
-                                 sc.n_zero, s.k0, f);
+    cudaError_t e = launch_det_begin(a, s, sc, f, one_sort, st);
     launches += 1;
     if (e != cudaSuccess || a.n_txns == 0) return e;
     const int G = a.max_ops <= 8 ? 8 : a.max_ops <= 16 ? 16 : 32;
@@ -467,15 +397,14 @@ cudaError_t fold_run(const ExecArgs& a, SortScratch& s, void* scratch, uint32_t&
     }
     if (e != cudaSuccess) return e;
     launches += 1;
-    return launch_after(det_finish, std::min<unsigned>(blocks_for(a.n_txns, RANK_TILE), 152u), 1024, st, a,
-                        s.work, sc.rank_desc);
+    return launch_det_finish(a, s, sc, st);
 }
 
 }  // namespace
 
 // (the version store of an MVCC batch shares this scratch: one 16-byte value per op)
 size_t fold_seg_bytes(size_t max_ops, size_t max_txns) {
-    return std::max<size_t>(max_ops * 16, fold_scratch(nullptr, max_ops, max_txns).n_zero * 16);
+    return std::max<size_t>(max_ops * 16, det_scratch(nullptr, max_ops, max_txns, CHUNK_LOG2, FT_TILE<16>).n_zero * 16);
 }
 
 cudaError_t det_fold_kv(const ExecArgs& a, uint32_t field_bytes, SortScratch& s, void* scratch,

@@ -362,6 +362,47 @@ struct ExecArgs {
 };
 
 
+// The last-name index: per district the customers sorted by (last, first,
+// number) with their last names beside them, and for the name ids below
+// NAME_PICKS, the range the workload draws from, the customer each selects
+// (row + 1, 0: nobody), so that most look-ups are one load.
+constexpr uint32_t NAME_PICKS = 1024, OE_CUSTOMERS = 3000;
+struct NameIndex {
+    const uint32_t* idx;
+    const int64_t* last;
+    const uint32_t* pick;
+#ifdef __CUDACC__
+    // First position in [lo, hi) whose name is not below `name` (upper: above).
+    static __device__ uint32_t bound(const int64_t* s, uint32_t lo, uint32_t hi, int64_t name, bool upper) {
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            const int64_t v = s[mid];
+            if (upper ? v <= name : v < name) lo = mid + 1; else hi = mid;
+        }
+        return lo;
+    }
+    // The customer row at position ceil(n / 2) among the district's n customers
+    // of that name, ~0u when there is none (or no such district).
+    __device__ uint32_t search(uint32_t district, int64_t name) const {
+        const uint32_t base = district * OE_CUSTOMERS;
+        const uint32_t lo = bound(last + base, 0, OE_CUSTOMERS, name, false);
+        const uint32_t hi = bound(last + base, lo, OE_CUSTOMERS, name, true);
+        return hi > lo ? base + idx[base + lo + (hi - lo + 1) / 2 - 1] : ~0u;
+    }
+    __device__ uint32_t customer(uint32_t W, uint32_t district, uint32_t name) const {
+        if (district >= 10u * W) return ~0u;
+        return name < NAME_PICKS ? pick[district * NAME_PICKS + name] - 1u : search(district, name);
+    }
+#endif
+};
+
+// Order-entry columns (table ids as in gcc_db_create) and the last-name index.
+struct OeTables {
+    uint64_t* c[24];
+    NameIndex names;
+};
+
+
 // Shared-memory staging per op: descriptor, observed word, value read, value
 // to write and one more word (TicToc's rts): the read and write sets live in
 // shared memory while the transaction runs, so aborted attempts never touch
@@ -479,13 +520,15 @@ gcc_status set_error(gcc_status s, const char* msg);
 size_t fold_seg_bytes(size_t max_ops, size_t max_txns);
 cudaError_t det_fold_kv(const ExecArgs& a, uint32_t field_bytes, SortScratch& s, void* scratch,
                         uint32_t& launches, cudaStream_t st);
-// Deterministic order-entry batch: each record's accesses applied in id order
-// by one warp over the sorted access table (reads, final records, NewOrder
-// inserts, results, dense ranks, batch counters).  `flags` holds 2 * n_txns
-// words, `heads` n_ops words; key_bits covers n_meta.
-cudaError_t det_serial_oe(const ExecArgs& a, SortScratch& s, uint32_t* scan_tmp, uint32_t* flags,
-                          uint32_t* heads, int key_bits, int sm_count, cudaStream_t st);
-int det_serial_oe_launches(int key_bits);
+// Deterministic order-entry batch by segmented prefix sums over the sorted
+// access table (reads, final records, NewOrder inserts, results, ranks, batch
+// counters).  `a.ops` as submitted (payments by last name unresolved);
+// `scratch` holds oe_scratch_bytes(max_batch_ops, max_batch_txns) bytes, `list`
+// n_ops words.  Begins the batch itself.
+struct OeTables;
+size_t oe_scratch_bytes(size_t max_ops, size_t max_txns);
+cudaError_t det_serial_oe(const ExecArgs& a, const OeTables& T, SortScratch& s, void* scratch,
+                          uint32_t* list, uint32_t& launches, cudaStream_t st);
 
 // OCC / TO: replace raw commit timestamps by dense ranks 0..committed-1.
 cudaError_t densify_commit_order(const ExecArgs& a, SortScratch& s, cudaStream_t st);
@@ -503,9 +546,10 @@ cudaError_t densify_tictoc(const ExecArgs& a, SortScratch& s, cudaStream_t st);
 // unknown kind, which makes its transaction invalid, when nobody has the
 // name).
 cudaError_t build_name_index(const int64_t* c_last, const int64_t* c_first, uint32_t n_districts,
-                             uint32_t* idx, int64_t* last_sorted, cudaStream_t st);
-cudaError_t resolve_by_name(const uint64_t* ops, uint64_t n, uint32_t W, const uint32_t* idx,
-                            const int64_t* last_sorted, uint64_t* out, cudaStream_t st);
+                             uint32_t* idx, int64_t* last_sorted, uint32_t* pick, cudaStream_t st);
+struct NameIndex;
+cudaError_t resolve_by_name(const uint64_t* ops, uint64_t n, uint32_t W, const NameIndex& names,
+                            uint64_t* out, cudaStream_t st);
 // MVCC, after the execute kernel: every slot's newest entry written into the
 // table, its version pointer cleared, every head word zeroed.
 cudaError_t launch_mv_flatten(const ExecArgs& a, uint32_t field_bytes, cudaStream_t st);

@@ -95,6 +95,7 @@ struct gcc_db {
     // batch's ops with by-name payments resolved
     uint32_t* name_idx = nullptr;
     int64_t* name_last = nullptr;
+    uint32_t* name_pick = nullptr;
     uint64_t* ops_resolved = nullptr;
     // latest execution
     cudaStream_t last_stream = nullptr;
