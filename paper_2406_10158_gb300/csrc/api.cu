@@ -149,6 +149,10 @@ void free_db(gcc_db* db) {
     cudaFree(db->fold_flags);
     cudaFree(db->fold_seg);
     cudaFree(db->mv_slot);
+    cudaFree(db->rank.bits);
+    cudaFree(db->rank.counts);
+    cudaFree(db->rank.desc);
+    cudaFree(db->rank.ticket);
     cudaFree(db->unit_cnt);
     cudaFree(db->unit_link);
     cudaFree(db->name_idx);
@@ -248,6 +252,12 @@ gcc_status create_impl(const gcc_db_desc* desc, gcc_db** out) {
     if ((s = dev_alloc(&db->fold_flags, d.max_batch_txns * 8, "validity flags and ranks")))
         return bail(s);
     if ((s = dev_alloc(reinterpret_cast<uint8_t**>(&db->fold_seg),
+    db->rank.words = (uint32_t)std::max<uint64_t>(d.max_batch_txns, 2048);
+    if ((s = dev_alloc(&db->rank.bits, db->rank.words * 4ull, "commit timestamp bits")) ||
+        (s = dev_alloc(&db->rank.counts, db->rank.words * 8ull, "commit timestamp counts")) ||
+        (s = dev_alloc(&db->rank.desc, gcc::rank_desc_words(db->rank.words) * 8, "rank descriptors")) ||
+        (s = dev_alloc(&db->rank.ticket, 4, "rank ticket")))
+        return bail(s);
                        d.schema == GCC_SCHEMA_KV
                            ? gcc::fold_seg_bytes(d.max_batch_ops, d.max_batch_txns)
                            : gcc::oe_scratch_bytes(d.max_batch_ops, d.max_batch_txns),
@@ -357,7 +367,6 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
     a.need = db->need;
     a.order_key = db->order_key;
     a.seq = db->fold_flags;
-    a.order_key_uses_base = scheme == GCC_OCC || scheme == GCC_TO;   // MVCC: batch-relative
     // MVCC version store: one entry per committed write, in scratch that
     // the commit ranks only need after the store has been flattened
     a.mv_wts = db->sort.k0;
@@ -480,8 +489,8 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
         launches += 1;                                       // flatten (+ a memset)
     }
     if (n_txns && (scheme == GCC_OCC || scheme == GCC_TO || scheme == GCC_MVCC)) {
-        GCC_CK(gcc::densify_commit_order(a, db->sort, st));
-        launches += 1 + gcc::radix_sort_launches(32) + 1;    // emit, sort, rank
+        GCC_CK(gcc::densify_commit_order(a, db->rank, scheme, st));
+        launches += 3;                                       // mark, scan, assign
     }
     if (n_txns && scheme == GCC_DET) {
         GCC_CK(gcc::densify_in_id_order(a, db->fold_flags, db->scan_tmp, st));

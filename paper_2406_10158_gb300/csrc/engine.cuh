@@ -328,7 +328,6 @@ struct ExecArgs {
     unsigned long long* order_key;// OCC/TO/TicToc: raw commit timestamp per txn
     uint32_t* seq;                // TicToc: commit sequence number per txn (ties)
     uint32_t det_all;             // DET dataflow: every access waits for all earlier ones
-    int order_key_uses_base;      // OCC: timestamps count from BatchState::ticket_base
     BatchState* st;
     DbState* dbs;
     // policy
@@ -530,8 +529,16 @@ size_t oe_scratch_bytes(size_t max_ops, size_t max_txns);
 cudaError_t det_serial_oe(const ExecArgs& a, const OeTables& T, SortScratch& s, void* scratch,
                           uint32_t* list, uint32_t& launches, cudaStream_t st);
 
-// OCC / TO: replace raw commit timestamps by dense ranks 0..committed-1.
-cudaError_t densify_commit_order(const ExecArgs& a, SortScratch& s, cudaStream_t st);
+// OCC / TO / MVCC: replace raw commit timestamps by dense ranks 0..committed-1.
+struct RankScratch {
+    uint32_t* bits;               // a bit per timestamp, zero between batches
+    uint64_t* counts;             // per word: bits before it << 32 | its bits
+    uint64_t* desc;               // look-back words of the scan, zero between batches
+    uint32_t* ticket;             // its tiles, zero between batches
+    uint32_t words;
+};
+size_t rank_desc_words(size_t words);
+cudaError_t densify_commit_order(const ExecArgs& a, const RankScratch& r, gcc_scheme scheme, cudaStream_t st);
 // Deterministic scheme run op by op: dense ranks in transaction-id order over
 // the committed transactions (`flags`: n_txns words, `scan_tmp`:
 // scan_tmp_words(n_txns) words).

@@ -502,7 +502,6 @@ gcc_status gcc_multi_plan_create(gcc_scheme scheme, const gcc_multi_batch* b, ui
         a.meta = db->meta;
         a.n_meta = db->n_meta;
         a.order_key = db->order_key;
-        a.order_key_uses_base = scheme != GCC_NO_WAIT_2PL;
         a.st = db->st;
         a.dbs = reinterpret_cast<gcc::DbState*>(reinterpret_cast<char*>(pl->d_ms) +
                                                 offsetof(gcc::MultiState, clock));
@@ -534,7 +533,6 @@ gcc_status gcc_multi_plan_create(gcc_scheme scheme, const gcc_multi_batch* b, ui
             a.max_ops = db->d.max_ops_per_txn;
             a.need = db->need;
             a.dbs = db->dbs;
-            a.order_key_uses_base = 0;
             continue;                    // control words are not used
         }
         // control words in a state this scheme can start from

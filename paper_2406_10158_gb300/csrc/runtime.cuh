@@ -83,6 +83,7 @@ struct gcc_db {
     MetaState meta_state = META_ZERO;
     // scratch
     gcc::SortScratch sort{};
+    gcc::RankScratch rank{};
     uint32_t* scan_tmp = nullptr;
     uint32_t* need = nullptr;
     unsigned long long* order_key = nullptr;
