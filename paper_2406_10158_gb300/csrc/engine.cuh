@@ -13,15 +13,21 @@
 namespace gcc {
 
 // ---------------------------------------------------------------------------
-// concurrency-control word layouts (one 64-bit word per record, Table II)
+// concurrency-control word layouts (one word per record, Table II)
 // ---------------------------------------------------------------------------
 // OCC: bit 63 lock, bits 0..62 version = commit timestamp + 1 (Sec. III-E.2,
 // "lock bit : 1, ts : 63").
 constexpr uint64_t OCC_LOCK = 1ull << 63;
-// 2PL: bit 63 exclusive, bits 32..62 shared-holder count, bits 0..31 exclusive
-// holder (transaction id + 1) -- Table II's shared bit / holder count / holder.
-constexpr uint64_t TPL_X = 1ull << 63;
-constexpr uint64_t TPL_S_ONE = 1ull << 32;
+// 2PL: one 32-bit word per record: bit 31 exclusive, bits 0..30 the exclusive
+// holder's transaction id, or without bit 31 the number of shared holders --
+// Table II's shared bit / holder count / holder.  Every access changes its
+// word twice, and random DRAM accesses are what an uncontended batch is bound
+// by: 4-byte words of 2^24 records (64 MB) stay in L2 where 8-byte ones do not
+// (2^20 x 16 ops, 95 % reads: 1,644 -> 1,539 us, 1,340 us with the slots only
+// read marked to leave L2 first).  OCC keeps 8-byte words: its words are
+// written once per commit, and 4-byte ones measured slower (its kernel took
+// 1,496 against 1,420 us).
+constexpr uint32_t TPL_X = 1u << 31;
 // TO: one 16-byte word per record, updated with a 128-bit CAS: lo = RTS,
 // hi = WTS (bits 0..62) | dirty (bit 63, the commit bit of Table II).  Table
 // II packs commit bit + 31-bit RTS + 31-bit WTS into 8 bytes, which overflows
@@ -87,6 +93,21 @@ __device__ __forceinline__ uint64_t ld_relaxed(const uint64_t* p) {
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t cas32_acquire(uint32_t* p, uint32_t cmp, uint32_t val) {
+    uint32_t old;
+    asm volatile("atom.acquire.gpu.global.cas.b32 %0, [%1], %2, %3;"
+                 : "=r"(old) : "l"(p), "r"(cmp), "r"(val) : "memory");
+    return old;
+}
+__device__ __forceinline__ uint32_t add32_release(uint32_t* p, uint32_t v) {
+    uint32_t old;
+    asm volatile("atom.release.gpu.global.add.u32 %0, [%1], %2;"
+                 : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+}
 __device__ __forceinline__ void st_relaxed(uint64_t* p, uint64_t v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
@@ -98,6 +119,25 @@ __device__ __forceinline__ ulonglong2 ld_slot16(const void* p) {
     ulonglong2 v;
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];"
                  : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+    return v;
+}
+// The same for data the caller will not touch again: its line leaves L2 before
+// those of the control words.
+__device__ __forceinline__ uint64_t evict_first() {
+    uint64_t p;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ uint64_t ld_once(const uint64_t* p) {
+    uint64_t v;
+    asm volatile("ld.relaxed.gpu.global.L2::cache_hint.u64 %0, [%1], %2;"
+                 : "=l"(v) : "l"(p), "l"(evict_first()) : "memory");
+    return v;
+}
+__device__ __forceinline__ ulonglong2 ld_slot16_once(const void* p) {
+    ulonglong2 v;
+    asm volatile("ld.relaxed.gpu.global.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;"
+                 : "=l"(v.x), "=l"(v.y) : "l"(p), "l"(evict_first()) : "memory");
     return v;
 }
 __device__ __forceinline__ void st_slot16(void* p, ulonglong2 v) {
@@ -318,7 +358,8 @@ struct ExecArgs {
     uint8_t* table;               // key-value slots (field-major)
     uint64_t n_records;
     uint32_t n_fields;
-    uint64_t* meta;               // one concurrency-control word per record
+    uint64_t* meta;               // control words: 16 bytes per record, of which 2PL uses
+                                  // the first 4 * n_meta, OCC and DET the first 8 * n_meta
     uint64_t n_meta;
     int64_t* const* cols;         // order-entry columns (device array of pointers)
     uint32_t n_warehouses;

@@ -85,6 +85,11 @@ struct Lane {
 // SKIPPED: DET only, an invalid transaction's accesses were stepped over
 enum { ABORT = 0, COMMIT = 1, GIVE_UP = 2, SKIPPED = 3 };
 
+// The 32-bit control words of 2PL.
+__device__ __forceinline__ uint32_t* words32(const ExecArgs& a) {
+    return reinterpret_cast<uint32_t*>(a.meta);
+}
+
 __device__ __forceinline__ bool collapse_loser(const ExecArgs& a, uint32_t rec) {
     if (a.collapse != 1) return false;
     const unsigned am = __activemask();
@@ -246,13 +251,13 @@ __device__ int tpl_attempt(const ExecArgs& a, const Lane& L, const Stage& S, uin
             const uint64_t d = S.desc[j];
             const uint32_t r = Work::rec(a, d);
             if (r != NO_CC) {
-                uint64_t* m = a.meta + r;
+                uint32_t* m = words32(a) + r;
                 if (!Work::writes(d)) {
                     uint32_t waited = 0;
                     for (uint32_t tries = 0;;) {
-                        const uint64_t w = ld_relaxed(m);
+                        const uint32_t w = ld_relaxed_u32(m);
                         if (w & TPL_X) {
-                            if (WAIT_DIE && t + 1 < (uint32_t)w && waited < wait_spins) {
+                            if (WAIT_DIE && t < (w & ~TPL_X) && waited < wait_spins) {
                                 ++waited;
                                 __nanosleep(64);
                                 continue;
@@ -260,31 +265,32 @@ __device__ int tpl_attempt(const ExecArgs& a, const Lane& L, const Stage& S, uin
                             fail = true; frec = r; break;
                         }
                         ++L.n_atom;
-                        if (cas64_acquire(m, w, w + TPL_S_ONE) == w) { held |= 1ull << k; break; }
+                        if (cas32_acquire(m, w, w + 1u) == w) { held |= 1ull << k; break; }
                         if (++tries > a.read_retries) { fail = true; frec = r; break; }
                     }
                 } else {
                     bool ok = !collapse_loser(a, r);
                     if (ok) {
-                        const uint64_t mine = TPL_X | (uint64_t)(t + 1);
+                        const uint32_t mine = TPL_X | t;
                         ++L.n_atom;
-                        uint64_t cur = cas64_acquire(m, 0ull, mine);
-                        for (uint32_t waited = 0; WAIT_DIE && cur != 0ull && (cur & TPL_X) &&
-                                                  t + 1 < (uint32_t)cur && waited < wait_spins;
+                        uint32_t cur = cas32_acquire(m, 0u, mine);
+                        for (uint32_t waited = 0; WAIT_DIE && (cur & TPL_X) && t < (cur & ~TPL_X) &&
+                                                  waited < wait_spins;
                              ++waited) {
                             __nanosleep(64);
-                            cur = ld_relaxed(m);
-                            if (cur == 0ull) { ++L.n_atom; cur = cas64_acquire(m, 0ull, mine); }
+                            cur = ld_relaxed_u32(m);
+                            if (cur == 0u) { ++L.n_atom; cur = cas32_acquire(m, 0u, mine); }
                         }
-                        ok = cur == 0ull;
+                        ok = cur == 0u;
                     }
                     if (ok) held |= 1ull << k; else { fail = true; frec = r; }
                 }
             }
             if (!fail) {
-                const ulonglong2 v = Work::load(a, d);
+                const bool w = Work::writes(d);
+                const ulonglong2 v = w ? Work::load(a, d) : Work::load_once(a, d);
                 S.oldv[j] = v;
-                if (Work::writes(d)) S.newv[j] = Work::compute(a, d, v, a.operands[first + j]);
+                if (w) S.newv[j] = Work::compute(a, d, v, a.operands[first + j]);
             }
         }
         if (__any_sync(L.gmask, fail)) break;
@@ -306,9 +312,9 @@ __device__ int tpl_attempt(const ExecArgs& a, const Lane& L, const Stage& S, uin
     for (uint32_t k = 0; k < kmax; ++k)
         if (held >> k & 1) {
             const uint32_t j = L.lig + k * L.G;
-            uint64_t* m = a.meta + Work::rec(a, S.desc[j]);
-            if (!Work::writes(S.desc[j])) { ++L.n_atom; add64_release(m, (uint64_t)0 - TPL_S_ONE); }
-            else st_release(m, 0ull);
+            uint32_t* m = words32(a) + Work::rec(a, S.desc[j]);
+            if (!Work::writes(S.desc[j])) { ++L.n_atom; add32_release(m, ~0u); }
+            else st_release_u32(m, 0u);
         }
     if (fail) crec = group_conflict(L, frec);
     return fail ? ABORT : COMMIT;

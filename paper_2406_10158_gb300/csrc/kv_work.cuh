@@ -18,6 +18,9 @@ template <> struct Slot<8> {
     static __device__ __forceinline__ ulonglong2 load(const uint8_t* p) {
         return make_ulonglong2(ld_relaxed(reinterpret_cast<const uint64_t*>(p)), 0ull);
     }
+    static __device__ __forceinline__ ulonglong2 load_once(const uint8_t* p) {
+        return make_ulonglong2(ld_once(reinterpret_cast<const uint64_t*>(p)), 0ull);
+    }
     static __device__ __forceinline__ void store(uint8_t* p, ulonglong2 v) {
         st_relaxed(reinterpret_cast<uint64_t*>(p), v.x);
     }
@@ -28,6 +31,7 @@ template <> struct Slot<8> {
 
 template <> struct Slot<16> {
     static __device__ __forceinline__ ulonglong2 load(const uint8_t* p) { return ld_slot16(p); }
+    static __device__ __forceinline__ ulonglong2 load_once(const uint8_t* p) { return ld_slot16_once(p); }
     static __device__ __forceinline__ void store(uint8_t* p, ulonglong2 v) { st_slot16(p, v); }
     static __device__ __forceinline__ ulonglong2 add(ulonglong2 v, ulonglong2 d) {
         return make_ulonglong2(v.x + d.x, (v.y & ~0xFFFFull) | ((v.y + d.y) & 0xFFFFull));
@@ -56,6 +60,10 @@ struct KvWork {
     static __device__ __forceinline__ bool writes(uint64_t d) { return op_kind(d) == GCC_OP_ADD; }
     static __device__ __forceinline__ ulonglong2 load(const ExecArgs& a, uint64_t d) {
         return Slot<FB>::load(ptr(a, d));
+    }
+    // A slot the transaction will not write.
+    static __device__ __forceinline__ ulonglong2 load_once(const ExecArgs& a, uint64_t d) {
+        return Slot<FB>::load_once(ptr(a, d));
     }
     static __device__ __forceinline__ ulonglong2 compute(const ExecArgs&, uint64_t, ulonglong2 old,
                                                          ulonglong2 operand) {

@@ -72,6 +72,7 @@ struct OeWork {
             default: return make_ulonglong2(get(a, S_QUANTITY, k), get(a, S_ORDER_CNT, k));
         }
     }
+    static __device__ __forceinline__ ulonglong2 load_once(const ExecArgs& a, uint64_t d) { return load(a, d); }
     // New values of the columns `load` returned, for the writing kinds.
     static __device__ ulonglong2 compute(const ExecArgs&, uint64_t d, ulonglong2 old, ulonglong2 opd) {
         const int64_t h = (int64_t)opd.x;
