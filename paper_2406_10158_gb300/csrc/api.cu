@@ -144,15 +144,15 @@ void free_db(gcc_db* db) {
     cudaFree(db->sort.v1);
     cudaFree(db->sort.work);
     cudaFree(db->scan_tmp);
+    cudaFree(db->rank.bits);
+    cudaFree(db->rank.counts);
+    cudaFree(db->rank.desc);
+    cudaFree(db->rank.ticket);
     cudaFree(db->need);
     cudaFree(db->order_key);
     cudaFree(db->fold_flags);
     cudaFree(db->fold_seg);
     cudaFree(db->mv_slot);
-    cudaFree(db->rank.bits);
-    cudaFree(db->rank.counts);
-    cudaFree(db->rank.desc);
-    cudaFree(db->rank.ticket);
     cudaFree(db->unit_cnt);
     cudaFree(db->unit_link);
     cudaFree(db->name_idx);
@@ -247,17 +247,17 @@ gcc_status create_impl(const gcc_db_desc* desc, gcc_db** out) {
         return bail(s);
     db->sort.err = &db->st->error;
     if ((s = dev_alloc(&db->scan_tmp, gcc::scan_tmp_words(items) * 4, "scan scratch"))) return bail(s);
-    if ((s = dev_alloc(&db->need, d.max_batch_ops * 4, "wait thresholds"))) return bail(s);
-    if ((s = dev_alloc(&db->order_key, d.max_batch_txns * 8, "commit keys"))) return bail(s);
-    if ((s = dev_alloc(&db->fold_flags, d.max_batch_txns * 8, "validity flags and ranks")))
-        return bail(s);
-    if ((s = dev_alloc(reinterpret_cast<uint8_t**>(&db->fold_seg),
     db->rank.words = (uint32_t)std::max<uint64_t>(d.max_batch_txns, 2048);
     if ((s = dev_alloc(&db->rank.bits, db->rank.words * 4ull, "commit timestamp bits")) ||
         (s = dev_alloc(&db->rank.counts, db->rank.words * 8ull, "commit timestamp counts")) ||
         (s = dev_alloc(&db->rank.desc, gcc::rank_desc_words(db->rank.words) * 8, "rank descriptors")) ||
         (s = dev_alloc(&db->rank.ticket, 4, "rank ticket")))
         return bail(s);
+    if ((s = dev_alloc(&db->need, d.max_batch_ops * 4, "wait thresholds"))) return bail(s);
+    if ((s = dev_alloc(&db->order_key, d.max_batch_txns * 8, "commit keys"))) return bail(s);
+    if ((s = dev_alloc(&db->fold_flags, d.max_batch_txns * 8, "validity flags and ranks")))
+        return bail(s);
+    if ((s = dev_alloc(reinterpret_cast<uint8_t**>(&db->fold_seg),
                        d.schema == GCC_SCHEMA_KV
                            ? gcc::fold_seg_bytes(d.max_batch_ops, d.max_batch_txns)
                            : gcc::oe_scratch_bytes(d.max_batch_ops, d.max_batch_txns),
