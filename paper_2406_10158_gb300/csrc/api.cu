@@ -78,7 +78,12 @@ gcc_exec_params defaults() {
 
 uint32_t queue_after_for(const gcc_exec_params& p, gcc_scheme scheme) {
     if (p.queue_after) return p.queue_after;
-    return scheme == GCC_OCC ? 64u : 16u;
+    // TicToc is optimistic as OCC is -- its aborts mostly mean that somebody
+    // committed -- and its queues serve one attempt at a time: 32 instead of 16
+    // takes ragged transactions at Zipf 0.6 from 12.7 to 8.2 ms and 2^20 x 16
+    // ops from 32.2 to 28.4 ms (Zipf 0.6) and 57.8 to 49.0 ms (0.8, 95 %
+    // reads); at 0.99 with half writes the queues are needed and 64 costs 7 %.
+    return scheme == GCC_OCC ? 64u : scheme == GCC_TICTOC ? 32u : 16u;
 }
 
 gcc_exec_params merged(const gcc_exec_params* in) {

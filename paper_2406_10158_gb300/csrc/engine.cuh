@@ -68,7 +68,7 @@ struct BatchState {
     unsigned long long atomics;      // global atomic operations of the execute kernel
     unsigned long long mv_used;      // MVCC: version-store entries taken
     unsigned int error;              // GCC_DEVERR_* bits
-    unsigned int pad;
+    unsigned int idle;               // lane groups that found no transaction left
 };
 
 // Retry queues per database (one 64-bit word each).

@@ -28,7 +28,7 @@ struct MultiState {
     DbState clock;                 // shared OCC / TO clock of the launch
     unsigned long long padded;     // fetch space: chunks rounded up to a power of two
     unsigned int chunk_bits;       // log2 of the number of chunks in it
-    unsigned int pad;
+    unsigned int idle;             // lane groups that found no transaction left
 };
 
 // Transactions are handed out in chunks of FETCH_CHUNK consecutive ids, the
@@ -97,6 +97,7 @@ struct MultiFetch {
         }
         return true;
     }
+    __device__ __forceinline__ uint32_t* idle() const { return &ms->idle; }
     __device__ __forceinline__ void done(const Lane&, const ExecArgs&, Counters&) {}
 };
 
@@ -130,6 +131,7 @@ __global__ void multi_begin(const ExecArgs* __restrict__ args, DbState* const* _
             to = max(to, own[i]->to_clock);
         }
         ms->fetch = 0;
+        ms->idle = 0;
         ms->clock.occ_clock = occ;
         ms->clock.to_clock = to;
     }
