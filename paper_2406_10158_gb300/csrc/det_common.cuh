@@ -13,7 +13,7 @@ namespace {
 
 // Words of SortScratch::work between the pass tickets and the histograms.
 // The first two are left at zero by the kernel that uses them.
-enum { DW_BEGIN_DONE = 8, DW_UNTILED_ACC, DW_UNTILED, DW_VALID_DONE, DW_FINISH_TICKET };
+enum { DW_BEGIN_DONE = 8, DW_UNTILED_ACC, DW_UNTILED, DW_FINISH_TICKET };
 
 constexpr uint32_t DET_SPIN_MAX = 1u << 21;
 
@@ -140,8 +140,13 @@ det_begin(const __grid_constant__ ExecArgs a, uint32_t* work, ulonglong2* zero, 
         work[DW_UNTILED] = bad;
         work[DW_UNTILED_ACC] = 0;
     }
-    if (bad)
-        for (uint64_t i = threadIdx.x; i < a.n_ops; i += 256) keys[i] = f.key(i, f.none, false);
+    if (!bad) return;
+    for (uint64_t i = threadIdx.x * 4ull; i < a.n_ops; i += 1024)
+        if (i + 4 <= a.n_ops)
+            *reinterpret_cast<uint4*>(keys + i) = make_uint4(f.key(i, f.none, false), f.key(i + 1, f.none, false),
+                                                             f.key(i + 2, f.none, false), f.key(i + 3, f.none, false));
+        else
+            for (uint64_t j = i; j < a.n_ops; ++j) keys[j] = f.key(j, f.none, false);
 }
 
 // Launches det_begin; with one sort for the whole batch (`one_sort`) it also
@@ -178,22 +183,34 @@ __device__ __forceinline__ void clear_digits(DigitHist* h) {
         for (int c = threadIdx.x; c < 256 * HIST_COPIES; c += 256) h[p][c] = 0;
 }
 
-// The block's histograms into the batch's.  Where the op ranges did not tile
-// the ops (DW_UNTILED) the counts would miss the ops outside every range: the
-// last block counts all keys instead.  Every block of the grid calls it.
-__device__ __forceinline__ void flush_digits(DigitHist* h, uint32_t* work, const uint32_t* keys,
-                                             uint64_t n, int bits, int passes, int digit_bits) {
-    const bool untiled = work[DW_UNTILED] != 0;
+// Writes an op's key and counts it.  Where the op ranges do not tile the ops
+// (DW_UNTILED) every op holds the key of no record already (det_begin), and may
+// be written by more than one transaction: the exchange tells which key the new
+// one replaces, so the counts stay those of the keys.
+__device__ __forceinline__ void put_key(const AccessKeys& f, DigitHist* h, uint32_t* keys, uint64_t op, uint32_t k,
+                                        bool tiled) {
+    if (tiled) {
+        keys[op] = k;
+    } else {
+        const uint32_t old = atomicExch(keys + op, k);
+        count_digits(h, old, f.bits, f.passes, f.digit_bits, ~0u);
+    }
+    count_digits(h, k, f.bits, f.passes, f.digit_bits);
+}
+
+// The block's histograms into the batch's; where the op ranges do not tile the
+// ops, block 0 also counts the keys det_begin wrote.  Every block calls it.
+__device__ __forceinline__ void flush_digits(const AccessKeys& f, DigitHist* h, uint32_t* work, uint64_t n,
+                                             bool tiled) {
     __syncthreads();
-    if (untiled) {
-        if (!last_block(work + DW_VALID_DONE)) return;
-        clear_digits(h);
-        __syncthreads();
-        for (uint64_t i = threadIdx.x; i < n; i += 256)
-            count_digits(h, *(volatile const uint32_t*)(keys + i), bits, passes, digit_bits);
+    if (!tiled && blockIdx.x == 0) {
+        const uint64_t len = 1ull << f.chunk_log2;
+        for (uint64_t o = threadIdx.x * len; o < n; o += 256 * len)
+            count_digits(h, f.key(o, f.none, false), f.bits, f.passes, f.digit_bits,
+                         (uint32_t)(n - o < len ? n - o : len));
         __syncthreads();
     }
-    for (int p = 0; p < passes; ++p) {
+    for (int p = 0; p < f.passes; ++p) {
         uint32_t c = 0;
 #pragma unroll
         for (int i = 0; i < HIST_COPIES; ++i) c += h[p][threadIdx.x * HIST_COPIES + i];

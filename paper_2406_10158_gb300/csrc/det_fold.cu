@@ -25,11 +25,13 @@
 // in chunks of consecutive positions, each starting from the table the one
 // before left.  A chunk's operands are gathered and its read values scattered
 // at random (sorted order against op order); cutting keeps the two within L2
-// (2^CHUNK_LOG2 ops: 32 MB each), where a batch of 2^24 ops at once would go
-// to DRAM sector by sector.  (Table accesses pay for it: a chunk touches the
-// table more sparsely.  On 2^24 ops over 2.5 GiB, chunks of 2^20 to 2^22 are
-// within 3 % and one chunk for all 5 % slower.)  The chunk number sorts in the
-// key's spare high bits, so the whole batch still takes one sort.
+// (2^CHUNK_LOG2 ops: 16 MB each), where a batch of 2^24 ops at once would go
+// to DRAM sector by sector.  Table accesses pay for it: a chunk touches the
+// table more sparsely.  2^24 ops over 2.5 GiB take 1,518 us in chunks of 2^21
+// and 1,635 us in chunks of 2^22; 64 databases at once take 6.58 ms in chunks
+// of 2^20, 6.85 of 2^21 and 7.17 of 2^22.  The chunk number sorts in the key's
+// spare high bits (so few of them may make the chunks larger), and the whole
+// batch still takes one sort.
 #include "det_common.cuh"
 
 namespace gcc {
@@ -42,7 +44,7 @@ constexpr int FT_THREADS = 256;
 template <int FB> constexpr int FT_ITEMS = FB == 16 ? 2 : 4;
 template <int FB> constexpr int FT_TILE = FT_THREADS * FT_ITEMS<FB>;
 constexpr int FT_WARPS = FT_THREADS / 32;
-constexpr int CHUNK_LOG2 = 21;
+constexpr int CHUNK_LOG2 = 20;
 // One sort handles at most 2^30 ops (30-bit digit counts, 31-bit positions);
 // longer batches are sorted and folded in that many at a time.
 constexpr int SORT_LOG2 = 30;
@@ -133,8 +135,7 @@ fold_validate(const __grid_constant__ ExecArgs a, const AccessKeys f, uint32_t* 
                 const uint64_t op = (uint64_t)first[u] + lig;
                 const uint32_t k = f.key(op, no ? f.none : d_field(d[u]) * (uint32_t)a.n_records + d_key(d[u]),
                                          !no && d_kind(d[u]) == GCC_OP_ADD);
-                keys[op] = k;
-                if (tiled) count_digits(h, k, f.bits, f.passes, f.digit_bits);
+                put_key(f, h, keys, op, k, tiled);
             }
             // the ops past the first G of a long or malformed transaction
             if (inside[u] && (bad[u] || nops[u] > G)) {
@@ -142,8 +143,7 @@ fold_validate(const __grid_constant__ ExecArgs a, const AccessKeys f, uint32_t* 
                     const uint64_t op = (uint64_t)first[u] + j;
                     const uint32_t k = f.key(op, no ? f.none : d_field(d2) * (uint32_t)a.n_records + d_key(d2),
                                              !no && d_kind(d2) == GCC_OP_ADD);
-                    keys[op] = k;
-                    if (tiled) count_digits(h, k, f.bits, f.passes, f.digit_bits);
+                    put_key(f, h, keys, op, k, tiled);
                 }
             }
             if (lig == 0 && tb + u < t_end) {
@@ -157,15 +157,20 @@ fold_validate(const __grid_constant__ ExecArgs a, const AccessKeys f, uint32_t* 
         atomicAdd(&a.st->invalid, (unsigned long long)invalid);
         atomicOr(&a.st->error, GCC_DEVERR_INVALID);
     }
-    flush_digits(h, work, keys, a.n_ops, f.bits, f.passes, f.digit_bits);
+    flush_digits(f, h, work, a.n_ops, tiled);
 }
 
 // --- fold -------------------------------------------------------------------
+// A slot's line is not read again soon: 64 of its 128 bytes are fetched (2^24
+// ops: 1,542 -> 1,518 us; not keeping it in L1 or marking it to leave L2 first
+// were slower, 1,598 us).
 template <int FB>
 __device__ __forceinline__ ulonglong2 slot_load(const ExecArgs& a, uint32_t slot) {
     const uint8_t* p = a.table + (uint64_t)slot * FB;
-    if (FB == 16) return *reinterpret_cast<const ulonglong2*>(p);
-    return make_ulonglong2(*reinterpret_cast<const uint64_t*>(p), 0ull);
+    ulonglong2 v = make_ulonglong2(0ull, 0ull);
+    if (FB == 16) asm volatile("ld.global.L2::64B.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+    else asm volatile("ld.global.L2::64B.u64 %0, [%1];" : "=l"(v.x) : "l"(p));
+    return v;
 }
 template <int FB>
 __device__ __forceinline__ ulonglong2 slot_plus(ulonglong2 v, Sum s) {

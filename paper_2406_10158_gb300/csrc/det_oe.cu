@@ -127,33 +127,28 @@ oe_validate(const __grid_constant__ ExecArgs a, const __grid_constant__ OeTables
             const uint64_t op0 = first[u];
             if (!bad[u] && lig < 3) {
                 const uint32_t k = f.key(op0 + lig, no ? f.none : hrec, !no && pay);
-                keys[op0 + lig] = k;
-                if (tiled) count_digits(h, k, f.bits, f.passes, f.digit_bits);
+                put_key(f, h, keys, op0 + lig, k, tiled);
             }
             if (line) {
                 const uint64_t op = op0 + 3 + 2 * lig;
                 const uint32_t ki = f.key(op, f.none, false);
                 const uint32_t ks = f.key(op + 1, no ? f.none : 30011u * W + op_key(stock[u]), false);
-                keys[op] = ki;
-                keys[op + 1] = ks;
                 if (!no) a.reads[op] = make_ulonglong2((uint64_t)T.c[I_PRICE][op_key(item[u])], 0ull);
-                if (tiled) {
-                    // the item reads' keys are all one but for the chunk: counted
-                    // once where the transaction lies in one chunk
-                    const uint32_t k0 = f.key(op0, f.none, false);
-                    if (k0 == f.key(op0 + nops[u] - 1, f.none, false)) {
-                        if (lig == 0) count_digits(h, k0, f.bits, f.passes, f.digit_bits, (nops[u] - 3) / 2);
-                    } else {
-                        count_digits(h, ki, f.bits, f.passes, f.digit_bits);
-                    }
-                    count_digits(h, ks, f.bits, f.passes, f.digit_bits);
+                // the item reads' keys are all one but for the chunk: counted
+                // once where the transaction lies in one chunk
+                const uint32_t k0 = f.key(op0, f.none, false);
+                if (tiled && k0 == f.key(op0 + nops[u] - 1, f.none, false)) {
+                    keys[op] = ki;
+                    if (lig == 0) count_digits(h, k0, f.bits, f.passes, f.digit_bits, (nops[u] - 3) / 2);
+                } else {
+                    put_key(f, h, keys, op, ki, tiled);
                 }
+                put_key(f, h, keys, op + 1, ks, tiled);
             }
             if (inside[u] && bad[u])
                 for (uint32_t j = lig; j < nops[u]; j += 16) {
                     const uint32_t k = f.key(op0 + j, f.none, false);
-                    keys[op0 + j] = k;
-                    if (tiled) count_digits(h, k, f.bits, f.passes, f.digit_bits);
+                    put_key(f, h, keys, op0 + j, k, tiled);
                 }
             if (lig == 0 && tb + u < t_end) {
                 a.results[tb + u] = no ? gcc_txn_result{GCC_TXN_INVALID, 0u, ~0ull}
@@ -166,7 +161,7 @@ oe_validate(const __grid_constant__ ExecArgs a, const __grid_constant__ OeTables
         atomicAdd(&a.st->invalid, (unsigned long long)invalid);
         atomicOr(&a.st->error, GCC_DEVERR_INVALID);
     }
-    flush_digits(h, work, keys, a.n_ops, f.bits, f.passes, f.digit_bits);
+    flush_digits(f, h, work, a.n_ops, tiled);
 }
 
 // --- fold -------------------------------------------------------------------
