@@ -80,10 +80,15 @@ uint32_t queue_after_for(const gcc_exec_params& p, gcc_scheme scheme) {
     if (p.queue_after) return p.queue_after;
     // TicToc is optimistic as OCC is -- its aborts mostly mean that somebody
     // committed -- and its queues serve one attempt at a time: 32 instead of 16
-    // takes ragged transactions at Zipf 0.6 from 12.7 to 8.2 ms and 2^20 x 16
-    // ops from 32.2 to 28.4 ms (Zipf 0.6) and 57.8 to 49.0 ms (0.8, 95 %
-    // reads); at 0.99 with half writes the queues are needed and 64 costs 7 %.
+    // takes ragged transactions at Zipf 0.6 from 12.8 to 8.5 ms and 2^20 x 16
+    // ops at 0.6 from 32.5 to 30.1 ms.  Where queues are long already (Zipf
+    // 0.99, half writes) they are needed from 16 aborts on, and joined then
+    // (QUEUE_LONG): 418 ms before and after, 428 without that.
     return scheme == GCC_OCC ? 64u : scheme == GCC_TICTOC ? 32u : 16u;
+}
+
+uint32_t queue_soon_for(const gcc_exec_params& p, gcc_scheme scheme) {
+    return !p.queue_after && scheme == GCC_TICTOC ? 16u : queue_after_for(p, scheme);
 }
 
 gcc_exec_params merged(const gcc_exec_params* in) {
@@ -399,6 +404,7 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
     a.det_all = p.det_dataflow == 2 ? 1u : 0u;
     a.queue_width = p.queue_width;
     a.queue_after = queue_after_for(p, scheme);
+    a.queue_soon = queue_soon_for(p, scheme);
 
     const bool kv = db->d.schema == GCC_SCHEMA_KV;
     // deterministic batches: every record chain by prefix sums (the pipelines
@@ -775,7 +781,10 @@ gcc_status gcc_batch_wait(gcc_batch* b, uint64_t timeout_ns, gcc_txn_result* res
         if (timeout_ns != UINT64_MAX && waited >= timeout_ns)
             return fail(GCC_ERR_TIMEOUT, "batch still running after %llu ns",
                         (unsigned long long)waited);
-        if (spin > 64) std::this_thread::sleep_for(std::chrono::microseconds(20));
+        // a batch of some milliseconds is polled without sleeping: a 20 us sleep
+        // lasts 70 us and more, as much as a small batch's kernel
+        if (waited > 4000000) std::this_thread::sleep_for(std::chrono::microseconds(20));
+        else if (spin > 64) std::this_thread::yield();
     }
     const cudaMemcpyKind k = outputs_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (results && b->n_txns)

@@ -630,13 +630,12 @@ __device__ __forceinline__ uint32_t mv_pointer(const ExecArgs& a, uint64_t d) {
     return e;
 }
 
-// The newest version of op d's slot older than ts: its entries from the
-// newest (version pointer e, read with acquire) down, else the table slot.
+// The newest version of a slot older than ts: its entries from the newest
+// (version pointer e, read with acquire) down, else the table slot's (`base`).
 // An entry's value is loaded beside its timestamp.  False when the walk would
 // step over more than MV_WALK_MAX entries (the attempt then aborts).
-template <class Work>
-__device__ __forceinline__ bool mv_version(const ExecArgs& a, uint64_t d, uint32_t ts, uint32_t e,
-                                           ulonglong2& out) {
+__device__ __forceinline__ bool mv_version(const ExecArgs& a, uint32_t ts, uint32_t e,
+                                           ulonglong2 base, ulonglong2& out) {
     for (uint32_t n = 0; e != 0; ++n) {
         if (n >= MV_WALK_MAX) return false;
         const uint32_t i = e - 1;
@@ -649,7 +648,7 @@ __device__ __forceinline__ bool mv_version(const ExecArgs& a, uint64_t d, uint32
         }
         e = nxt;
     }
-    out = Work::load(a, d);
+    out = base;
     return true;
 }
 
@@ -726,6 +725,9 @@ __device__ int mvcc_attempt(const ExecArgs& a, const Lane& L, const Stage& S, ui
             const uint32_t r = Work::rec(a, d);
             ulonglong2* m = heads + r;
             if (!Work::writes(d)) {
+                // the table slot, never written during the batch, beside the head:
+                // most slots have no entry and this is the version read
+                const ulonglong2 base = Work::load_once(a, d);
                 bool ok = false;
                 for (uint32_t tries = 0; tries <= a.read_retries; ++tries) {
                     const ulonglong2 h = ld128_acquire(m);
@@ -740,12 +742,14 @@ __device__ int mvcc_attempt(const ExecArgs& a, const Lane& L, const Stage& S, ui
                         const ulonglong2 o = cas128_acquire(m, h, make_ulonglong2(mv_pack(wts, ts), h.y));
                         if (o.x != h.x || o.y != h.y) continue;
                     }
-                    ok = mv_version<Work>(a, d, ts, pe, S.oldv[j]);
+                    ok = mv_version(a, ts, pe, base, S.oldv[j]);
                     break;
                 }
                 if (!ok) { fail = true; frec = r; }
             } else {
                 bool ok = !collapse_loser(a, r);
+                const ulonglong2 base = Work::load(a, d);
+                const ulonglong2 opd = a.operands[first + j];
                 for (uint32_t tries = 0; ok && tries <= a.read_retries; ++tries) {
                     const ulonglong2 h = ld128_acquire(m);
                     const uint32_t wts = mv_lo(h.x), rts = mv_hi(h.x), pend = mv_lo(h.y);
@@ -756,7 +760,7 @@ __device__ int mvcc_attempt(const ExecArgs& a, const Lane& L, const Stage& S, ui
                     // from h succeeds
                     uint32_t pe;
                     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(pe) : "l"(mv_slot_ptr(a, d)) : "memory");
-                    const ulonglong2 v = pe ? ld_slot16(a.mv_val + (pe - 1)) : Work::load(a, d);
+                    const ulonglong2 v = pe ? ld_slot16(a.mv_val + (pe - 1)) : base;
                     ++L.n_atom;
                     const ulonglong2 o = cas128_acquire(m, h, make_ulonglong2(h.x, mv_pack(ts, mv_hi(h.y))));
                     if (o.x != h.x || o.y != h.y) {
@@ -767,7 +771,7 @@ __device__ int mvcc_attempt(const ExecArgs& a, const Lane& L, const Stage& S, ui
                     S.obs[j] = pe;                              // the entry it supersedes
                     S.aux[j] = h.x;                             // the head's first word as installed
                     S.oldv[j] = v;
-                    S.newv[j] = Work::compute(a, d, v, a.operands[first + j]);
+                    S.newv[j] = Work::compute(a, d, v, opd);
                     break;
                 }
                 if (!ok) { fail = true; frec = r; }
@@ -934,6 +938,9 @@ constexpr uint64_t IDLE_LOOK_NS = 8000, IDLE_TURN_NS = 1000;
 // Admitted transactions always finish their attempt, so a queue never stalls;
 // a transaction still waiting at the kernel deadline gives up and abandons its
 // ticket, and the words are zeroed before every batch.
+// A TicToc transaction joins a queue of at least this many waiting after
+// queue_soon aborts already.
+constexpr int32_t QUEUE_LONG = 8;
 constexpr uint32_t NO_Q = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t queue_of(const ExecArgs& a, uint32_t rec) {
@@ -987,6 +994,9 @@ struct SingleFetch {
 template <int SCHEME, class Work, class Fetch>
 __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, uint64_t deadline,
                            Counters& c) {
+    // OCC's batches end without the wait (an abort there mostly means a commit),
+    // and its contended ones ran 2 % slower with the look
+    constexpr bool CUT_WAITS = SCHEME != GCC_OCC && SCHEME != GCC_DET;
     constexpr bool DENSE =
         SCHEME == GCC_NO_WAIT_2PL || SCHEME == GCC_2PL_WAIT_DIE || SCHEME == GCC_DET;
     bool finished = false, has = false, served = false;
@@ -1006,7 +1016,7 @@ __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, 
         if (!has && !finished) {
             if (!F.next(L, t, A)) {
                 finished = true;
-                if (L.lig == 0) atomicAdd(F.idle(), 1u);
+                if (CUT_WAITS && L.lig == 0) atomicAdd(F.idle(), 1u);
             } else {
                 const ExecArgs& a = *A;
                 const gcc_txn tx = a.txns[t];
@@ -1149,8 +1159,15 @@ __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, 
                     // transactions that keep aborting each other), then the
                     // queue of the record it conflicted on
                     wake = t2 + backoff_ns(a, t, attempts);
-                    if (a.rq && crec != NO_CC && attempts >= a.queue_after)
+                    if (a.rq && crec != NO_CC && attempts >= a.queue_after) {
                         pq = queue_of(a, crec);
+                    } else if (SCHEME == GCC_TICTOC && a.rq && crec != NO_CC && attempts >= a.queue_soon) {
+                        // not yet: only a queue that is already long
+                        uint64_t w = 0;
+                        if (L.lig == 0) w = ld_relaxed(a.rq + queue_of(a, crec));
+                        w = __shfl_sync(L.gmask, w, L.gbase);
+                        if ((int32_t)((uint32_t)(w >> 32) - (uint32_t)w) >= QUEUE_LONG) pq = queue_of(a, crec);
+                    }
                 }
             }
             if (outcome == COMMIT) {
@@ -1183,7 +1200,7 @@ __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, 
         // earliest wake-up (32 ns .. 1 us)
         if (!__any_sync(0xffffffffu, go)) {
             const uint64_t wnow = __shfl_sync(0xffffffffu, now, 0);     // the same on every lane
-            if (wnow >= look) {
+            if (CUT_WAITS && wnow >= look) {
                 const uint32_t groups = gridDim.x * (blockDim.x / L.G);
                 const uint32_t busy = groups - __shfl_sync(0xffffffffu, L.lane == 0 ? ld_relaxed_u32(F.idle()) : 0u, 0);
                 look = wnow + (busy == groups ? 4 * IDLE_LOOK_NS : IDLE_LOOK_NS);
