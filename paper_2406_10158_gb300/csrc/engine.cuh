@@ -493,13 +493,18 @@ struct SortScratch {
 constexpr int SORT_MAX_PASSES = 4;
 constexpr size_t SORT_HIST = 64;
 constexpr size_t SORT_DESC = SORT_HIST + SORT_MAX_PASSES * 256;
-// Items per tile: few enough per thread that a small sort still covers the
-// SMs, many for the large ones (order.cu gives the measurements).
+// Items per thread of a sort tile: few enough that a small sort still covers the
+// SMs, many for the large ones, whose tiles look back less often.  (Whole
+// deterministic batches: 2^16 ops 42.3 us with 4, 44.2 with 8; 2^18 ops 60.4
+// and 56.7; 2^19 ops 68.9 and 64.5; 2^20 ops 90.2 with 8 and 85.1 with 16.)
 constexpr int SORT_BLOCK = 256;
-constexpr int SORT_ITEMS_SMALL = 4, SORT_ITEMS_LARGE = 16;
-constexpr size_t SORT_SMALL = size_t(1) << 19;
+constexpr int SORT_ITEMS_SMALL = 4, SORT_ITEMS_MID = 8, SORT_ITEMS_LARGE = 16;
+constexpr size_t SORT_SMALL = size_t(1) << 17, SORT_MID = size_t(1) << 19;
+constexpr int sort_items(size_t n) {
+    return n <= SORT_SMALL ? SORT_ITEMS_SMALL : n <= SORT_MID ? SORT_ITEMS_MID : SORT_ITEMS_LARGE;
+}
 constexpr size_t sort_tiles(size_t n) {
-    const size_t tile = SORT_BLOCK * (n <= SORT_SMALL ? SORT_ITEMS_SMALL : SORT_ITEMS_LARGE);
+    const size_t tile = (size_t)SORT_BLOCK * sort_items(n);
     return (n + tile - 1) / tile;
 }
 // Words of one descriptor area: 256 per tile, 64-bit where a digit's count may
@@ -510,7 +515,9 @@ constexpr size_t sort_desc_words(size_t n) {
 constexpr size_t sort_work_words(size_t max_items) {
     const size_t a = sort_desc_words(max_items);
     const size_t b = sort_desc_words(max_items < SORT_SMALL ? max_items : SORT_SMALL);
-    return SORT_DESC + 2 * (a > b ? a : b);
+    const size_t c = sort_desc_words(max_items < SORT_MID ? max_items : SORT_MID);
+    const size_t ab = a > b ? a : b;
+    return SORT_DESC + 2 * (ab > c ? ab : c);
 }
 struct SortPlan {                 // digits of a sort on the low `bits` bits
     int passes, digit_bits;

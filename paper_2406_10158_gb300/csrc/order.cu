@@ -293,6 +293,8 @@ cudaError_t rs_run(SortScratch& s, uint32_t* keys, uint32_t* vals, size_t n, int
                    uint32_t** keys_out, uint32_t** vals_out, cudaStream_t st) {
     if (n <= SORT_SMALL)
         return rs_passes<uint32_t, SORT_ITEMS_SMALL>(s, keys, vals, n, bits, flagged, keys_out, vals_out, st);
+    if (n <= SORT_MID)
+        return rs_passes<uint32_t, SORT_ITEMS_MID>(s, keys, vals, n, bits, flagged, keys_out, vals_out, st);
     if (n < (size_t(1) << 30))
         return rs_passes<uint32_t, SORT_ITEMS_LARGE>(s, keys, vals, n, bits, flagged, keys_out, vals_out, st);
     return rs_passes<uint64_t, SORT_ITEMS_LARGE>(s, keys, vals, n, bits, flagged, keys_out, vals_out, st);
