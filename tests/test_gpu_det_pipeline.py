@@ -37,13 +37,15 @@ def make(nrec, nf, fb, **kw):
     return table, wl.kv_batch(7, nrec=nrec, nfields=nf, field_bytes=fb, **kw)
 
 
-# op counts around the fold's tiles (512 and 1,024), the sort's small tile (1,024), the switch to large
-# sort tiles (2^19) and a fold chunk (2^21); record counts down to one hot record, up to a power of two
+# op counts around the fold's tiles (512 and 1,024), the sort's tiles (1,024 and 2,048), the switches to
+# larger tiles (2^17, 2^19) and a fold chunk (2^20); record counts down to one hot record, up to a power of
+# two, and slot counts whose sort keys take digits of more than 8 bits (17 to 20 and 25 to 30 bits)
 @pytest.mark.parametrize("fb", [8, 16])
 @pytest.mark.parametrize("n,nrec,nf", [
     (1, 1, 1), (511, 1, 1), (513, 2, 3), (1023, 1024, 1), (1024, 1000, 2), (1025, 3, 1), (4097, 1, 2),
-    ((1 << 19) - 1, 4096, 4), (1 << 19, 7, 1), ((1 << 19) + 1, 1 << 16, 3),
-    ((1 << 21) - 1, 1 << 18, 4), ((1 << 21) + 1, 5, 1), ((1 << 22) + 4097, 1 << 12, 10)])
+    (1 << 17, 1 << 16, 8), ((1 << 17) + 1, 1 << 17, 1), (2049, 1 << 24, 1), (60000, (1 << 22) + 1, 10),
+    ((1 << 18) + 77, (1 << 25) - 1, 1), ((1 << 19) - 1, 4096, 4), (1 << 19, 7, 1), ((1 << 19) + 1, 1 << 16, 3),
+    ((1 << 20) + 1, 3, 1), ((1 << 21) - 1, 1 << 18, 4), ((1 << 21) + 1, 5, 1), ((1 << 22) + 4097, 1 << 12, 10)])
 def test_tile_and_chunk_edges(eng, n, nrec, nf, fb):
     table, batch = make(nrec, nf, fb, n_txns=n, ops_per_txn=1, theta=0.6 if nrec > 8 else 0.0)
     (res, reads, stats), final = run(eng, table, batch, fb, 1)
