@@ -66,11 +66,16 @@ __device__ __forceinline__ Sum sum_add(Sum a, Sum b) { return Sum{a.lo + b.lo, (
 // per group at once so that their headers and descriptors load together.
 // Every block takes one contiguous range of transactions.  Bound by the
 // shared-memory histogram updates (one per op and pass): 2^20 transactions of
-// 16 ops take 212 us, of which the stream of descriptors in and keys out would
+// 16 ops take 151 us, of which the stream of descriptors in and keys out would
 // take 35; a warp per transaction with every pair of keys compared took 256
 // without the histograms, and the sort's own histogram kernels 345 more.
+// Equal keys: groups of 8 and 16 lanes compare by rotation (the batch 1,520 ->
+// 1,459 us against __match_any_sync, which finds one distinct key at a time);
+// for 32 lanes the 16 rotations take too many registers (64 databases of up to
+// 64 ops: 6,900 us against 6,573), and 4 blocks on an SM hide the match's
+// latency better than 3 (6,573 against 6,795; 5 spill, 6,606).
 template <int G>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, G == 32 ? 4 : 1)
 fold_validate(const __grid_constant__ ExecArgs a, const AccessKeys f, uint32_t* __restrict__ keys,
               uint32_t* work, uint32_t per_block) {
     constexpr int GROUPS = 256 / G, U = G == 32 ? 2 : 4;
@@ -111,8 +116,18 @@ fold_validate(const __grid_constant__ ExecArgs a, const AccessKeys f, uint32_t* 
                         (d_kind(d[u]) != GCC_OP_READ && d_kind(d[u]) != GCC_OP_ADD);
             // equal keys among the group's lanes
             const unsigned holders = __ballot_sync(0xffffffffu, has);
-            const unsigned peers = __match_any_sync(0xffffffffu, d_key(d[u]));
-            if (has && __popc(peers & holders & gmask) > 1) wrong = true;
+            if constexpr (G <= 16) {
+                // every two lanes of the group meet in one of G / 2 rotations
+#pragma unroll
+                for (int o = 1; o <= G / 2; ++o) {
+                    const int other = gbase | ((lig + o) & (G - 1));
+                    const uint32_t k = __shfl_sync(0xffffffffu, d_key(d[u]), other);
+                    if (has && (holders >> other & 1u) && k == d_key(d[u])) wrong = true;
+                }
+            } else {
+                const unsigned peers = __match_any_sync(0xffffffffu, d_key(d[u]));
+                if (has && __popc(peers & holders) > 1) wrong = true;
+            }
             uint64_t d2 = 0;
             if constexpr (G == 32) {
                 if (!bad[u] && nops[u] > 32) {           // uniform over the warp

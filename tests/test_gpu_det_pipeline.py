@@ -107,6 +107,27 @@ def test_invalid_and_left_out(eng, n_txns, ops_range):
     assert np.array_equal(reads[pos.astype(np.int64)], ref_reads) and np.array_equal(final, ref)
 
 
+@pytest.mark.parametrize("k", [2, 7, 8, 15, 16, 17, 32, 33, 64])
+def test_every_pair_of_equal_keys(eng, k):
+    """A transaction of k ops for every two positions that share a key (record 0 among them, the value of
+    an empty lane's descriptor): each is invalid, and the distinct one after it commits."""
+    pairs = [(i, j) for i in range(k) for j in range(i + 1, k)]
+    n = 2 * len(pairs)
+    nrec = 101
+    table, batch = make(nrec, 2, 8, n_txns=n, ops_range=(k, k), theta=0.0)
+    keys = (np.arange(k)[None, :] + np.arange(n)[:, None] * 7) % nrec
+    for p, (i, j) in enumerate(pairs):
+        keys[2 * p, j] = keys[2 * p, i]
+    batch.ops["key"] = keys.reshape(-1)
+    (res, reads, stats), final = run(eng, table, batch, 8, k)
+    good = np.arange(1, n, 2)
+    ref, ref_reads = oracle.serial(table, wl.select(batch, good))
+    assert (res["status"][::2] == 3).all() and (res["status"][good] == oracle.ST_COMMITTED).all()
+    assert stats["invalid"] == len(pairs) and stats["committed"] == len(pairs)
+    assert np.array_equal(reads.reshape(n, k, -1)[good].reshape(ref_reads.shape), ref_reads)
+    assert np.array_equal(final, ref)
+
+
 def test_slot_ids_of_32_bits(eng):
     """2^31 slots and more leave no spare bit in the sort key: reads of two batches in turn against the
     closed form of the seeded table."""
