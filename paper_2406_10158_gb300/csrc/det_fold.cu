@@ -66,7 +66,7 @@ __device__ __forceinline__ Sum sum_add(Sum a, Sum b) { return Sum{a.lo + b.lo, (
 // per group at once so that their headers and descriptors load together.
 // Every block takes one contiguous range of transactions.  Bound by the
 // shared-memory histogram updates (one per op and pass): 2^20 transactions of
-// 16 ops take 151 us, of which the stream of descriptors in and keys out would
+// 16 ops take about 150 us, of which the stream of descriptors in and keys out would
 // take 35; a warp per transaction with every pair of keys compared took 256
 // without the histograms, and the sort's own histogram kernels 345 more.
 // Equal keys: groups of 8 and 16 lanes compare by rotation (the batch 1,520 ->

@@ -995,8 +995,13 @@ template <int SCHEME, class Work, class Fetch>
 __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, uint64_t deadline,
                            Counters& c) {
     // OCC's batches end without the wait (an abort there mostly means a commit),
-    // and its contended ones ran 2 % slower with the look
-    constexpr bool CUT_WAITS = SCHEME != GCC_OCC && SCHEME != GCC_DET;
+    // and its contended ones ran 2 % slower with the look.  TO gained 12 % on a
+    // read-mostly batch (2^20 x 16 ops, Zipf 0.6: 4.85 -> 4.25 ms) and lost 2 %
+    // with half writes (27.1 -> 27.7) and 4 % at Zipf 0.8 (351 -> 367), however
+    // seldom it looked: the code alone lengthens each link of the hot chain.
+    // The others gain more (MVCC 3.45 -> 2.30 ms, TicToc and 2PL 10 to 18 %
+    // read-mostly) than they lose at Zipf 0.8 (TicToc 5 %, 2PL 1 %, MVCC 2 %).
+    constexpr bool CUT_WAITS = SCHEME != GCC_OCC && SCHEME != GCC_TO && SCHEME != GCC_DET;
     constexpr bool DENSE =
         SCHEME == GCC_NO_WAIT_2PL || SCHEME == GCC_2PL_WAIT_DIE || SCHEME == GCC_DET;
     bool finished = false, has = false, served = false;
@@ -1199,17 +1204,20 @@ __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, 
         // 3. a warp where nobody attempted this round sleeps until its
         // earliest wake-up (32 ns .. 1 us)
         if (!__any_sync(0xffffffffu, go)) {
-            const uint64_t wnow = __shfl_sync(0xffffffffu, now, 0);     // the same on every lane
-            if (CUT_WAITS && wnow >= look) {
-                const uint32_t groups = gridDim.x * (blockDim.x / L.G);
-                const uint32_t busy = groups - __shfl_sync(0xffffffffu, L.lane == 0 ? ld_relaxed_u32(F.idle()) : 0u, 0);
-                look = wnow + (busy == groups ? 4 * IDLE_LOOK_NS : IDLE_LOOK_NS);
-                if (has) {
-                    const uint64_t most = (uint64_t)busy * IDLE_TURN_NS << (cuts < 20 ? cuts : 20);
-                    if (wake > wnow + most) {
-                        wake = wnow + mix64(A->seed ^ ((uint64_t)t << 32) ^ attempts) % (most + 1);
-                        if (cut_at != attempts) ++cuts;
-                        cut_at = attempts;
+            if constexpr (CUT_WAITS) {
+                const uint64_t wnow = __shfl_sync(0xffffffffu, now, 0);     // the same on every lane
+                if (wnow >= look) {
+                    const uint32_t groups = gridDim.x * (blockDim.x / L.G);
+                    const uint32_t busy =
+                        groups - __shfl_sync(0xffffffffu, L.lane == 0 ? ld_relaxed_u32(F.idle()) : 0u, 0);
+                    look = wnow + (busy == groups ? 4 * IDLE_LOOK_NS : IDLE_LOOK_NS);
+                    if (has) {
+                        const uint64_t most = (uint64_t)busy * IDLE_TURN_NS << (cuts < 20 ? cuts : 20);
+                        if (wake > wnow + most) {
+                            wake = wnow + mix64(A->seed ^ ((uint64_t)t << 32) ^ attempts) % (most + 1);
+                            if (cut_at != attempts) ++cuts;
+                            cut_at = attempts;
+                        }
                     }
                 }
             }
