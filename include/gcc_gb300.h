@@ -217,10 +217,9 @@ typedef struct gcc_exec_params {
                                   once [1] */
     uint32_t queue_after;      /* aborts of a transaction before it uses retry
                                   queues; 1 = from its first abort [2PL, TO,
-                                  MVCC: 16; TicToc: 32, or 16 where the
-                                  record's queue is already long; OCC: 64 --
-                                  an OCC abort nearly always means another
-                                  transaction committed, so its retries rarely
+                                  MVCC: 16; TicToc: 32; OCC: 64 -- an abort of
+                                  these two nearly always means another
+                                  transaction committed, so retries rarely
                                   need queueing] */
     uint32_t group_commit;     /* OCC on key-value databases: transactions per
                                   commit unit, 2..8 (1 = off) [1].  The

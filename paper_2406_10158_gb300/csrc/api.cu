@@ -80,15 +80,10 @@ uint32_t queue_after_for(const gcc_exec_params& p, gcc_scheme scheme) {
     if (p.queue_after) return p.queue_after;
     // TicToc is optimistic as OCC is -- its aborts mostly mean that somebody
     // committed -- and its queues serve one attempt at a time: 32 instead of 16
-    // takes ragged transactions at Zipf 0.6 from 12.8 to 8.5 ms and 2^20 x 16
-    // ops at 0.6 from 32.5 to 30.1 ms.  Where queues are long already (Zipf
-    // 0.99, half writes) they are needed from 16 aborts on, and joined then
-    // (QUEUE_LONG): 418 ms before and after, 428 without that.
+    // takes ragged transactions at Zipf 0.6 from 11.4 to 8.0 ms and 2^20 x 16
+    // ops from 30.9 to 26.4 ms at Zipf 0.6, from 57.7 to 47.8 at 0.8 with 95 %
+    // reads; within 2 % of each other at 0.8 and 0.99 with half writes.
     return scheme == GCC_OCC ? 64u : scheme == GCC_TICTOC ? 32u : 16u;
-}
-
-uint32_t queue_soon_for(const gcc_exec_params& p, gcc_scheme scheme) {
-    return !p.queue_after && scheme == GCC_TICTOC ? 16u : queue_after_for(p, scheme);
 }
 
 gcc_exec_params merged(const gcc_exec_params* in) {
@@ -396,7 +391,7 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
     a.read_retries = p.read_retries;
     a.inject_ppm = p.inject_abort_ppm;
     a.wait_budget_ns = p.wait_budget_ns;
-    a.deadline_ns = p.deadline_ns;
+    a.deadline_ns = std::min<uint64_t>(p.deadline_ns, gcc::DEADLINE_MAX_NS);
     a.seed = p.seed;
     a.rq = (p.retry_queue == 2 || p.immediate_restart) ? nullptr : db->rq;
     a.rq_mask = gcc::RETRY_QUEUES - 1;
@@ -404,7 +399,6 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
     a.det_all = p.det_dataflow == 2 ? 1u : 0u;
     a.queue_width = p.queue_width;
     a.queue_after = queue_after_for(p, scheme);
-    a.queue_soon = queue_soon_for(p, scheme);
 
     const bool kv = db->d.schema == GCC_SCHEMA_KV;
     // deterministic batches: every record chain by prefix sums (the pipelines

@@ -345,6 +345,9 @@ inline cudaError_t launch_after(void (*k)(P...), unsigned grid, unsigned block, 
 // ---------------------------------------------------------------------------
 // kernel arguments
 // ---------------------------------------------------------------------------
+// Longest kernel deadline that is told apart from a later one (19 hours).
+constexpr uint64_t DEADLINE_MAX_NS = 1ull << 46;
+
 struct ExecArgs {
     // batch
     const gcc_txn* txns;
@@ -388,7 +391,6 @@ struct ExecArgs {
     uint32_t queue_turn_ns;     // estimated time per queue turn
     uint32_t queue_width;       // tickets a queue admits at once
     uint32_t queue_after;       // aborts before a transaction uses the queues
-    uint32_t queue_soon;        // aborts before it joins one that is already long
     // MVCC version store of the batch: entry i = (wts, next, record, field,
     // value); capacity n_ops (one entry per committed write)
     uint32_t* mv_wts;

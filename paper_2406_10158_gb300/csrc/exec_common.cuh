@@ -58,6 +58,8 @@
 //   commit_step(a, L, S, t, first, nops) (work after commit, e.g. inserts).
 #pragma once
 
+#include <type_traits>
+
 #include "engine.cuh"
 
 namespace gcc {
@@ -900,6 +902,11 @@ __device__ void det_skip(const ExecArgs& a, const Lane& L, uint64_t first, uint3
 // backoff_cap_ns / backoff_base_ns.  Waits are deadlines on the global timer,
 // not round counts: a round lasts a few hundred nanoseconds in an idle warp
 // and several microseconds in a busy one.
+// MUL: the number by a multiplication, which takes fewer registers than the
+// 64-bit remainder, for the kernels that are short of them (TicToc, MVCC); 2PL
+// wait-die ran 1 % faster with it at Zipf 0.8 (425 -> 422 ms) and 3 % slower
+// at 0.6 (29.9 -> 30.9).
+template <bool MUL = false>
 __device__ __forceinline__ uint64_t backoff_ns(const ExecArgs& a, uint32_t t, uint32_t attempts) {
     if (a.backoff_base_ns == 0) return 0;
     uint64_t cap = a.backoff_cap_ns / a.backoff_base_ns;
@@ -907,15 +914,16 @@ __device__ __forceinline__ uint64_t backoff_ns(const ExecArgs& a, uint32_t t, ui
     const uint32_t sh = attempts - 1 < 20 ? attempts - 1 : 20;
     uint64_t window = 1ull << sh;
     if (window > cap) window = cap;
-    return (mix64(a.seed ^ ((uint64_t)t << 24) ^ attempts) % (window + 1)) * a.backoff_base_ns;
+    const uint64_t r = mix64(a.seed ^ ((uint64_t)t << 24) ^ attempts);
+    return (MUL ? __umul64hi(r, window + 1) : r % (window + 1)) * a.backoff_base_ns;
 }
 
 // The end of a batch.  A window of up to backoff_cap_ns spreads the attempts of
 // thousands of contenders; once the last transactions have been handed out
 // there are fewer and fewer, and a batch would end with a handful sitting out
 // windows of a millisecond with nobody left to collide with.  So a waiting
-// warp looks every IDLE_LOOK_NS (every four of them while all are) how many
-// lane groups are still at work, and waits a random part of at most
+// warp looks every IDLE_LOOK_NS (every 16 of them while all are) how many
+// lane groups are still at work, and backs off for a random part of at most
 // IDLE_TURN_NS for each of them: with so few contenders that leaves about a
 // turn each.  Long transactions that all conflict need more, so the bound
 // doubles with every attempt of a transaction that was cut short and aborted
@@ -923,7 +931,17 @@ __device__ __forceinline__ uint64_t backoff_ns(const ExecArgs& a, uint32_t t, ui
 // on 512 records).  Read-mostly MVCC batch of 2^18 transactions, Zipf 0.6:
 // 3.54 ms without, 2.27 with (2.80 at 4 us a group); looking every 2 us
 // instead of 8 slowed contended batches by 3 %.
+// The look's state takes two registers, the transaction counter and the deadline
+// one each instead of two, because every register it takes from the attempts
+// lengthens each link of a hot record's chain: with six for the look TicToc
+// took 403 ms for 2^20 x 16 ops at Zipf 0.8 and half writes, with two 379
+// (385 with no look at all), MVCC 514 and 495, 2PL wait-die 427 and 425.
 constexpr uint64_t IDLE_LOOK_NS = 8000, IDLE_TURN_NS = 1000;
+// The schemes that cut.  OCC's batches end without the wait (an abort there
+// mostly means a commit); TO gained 12 % on a read-mostly batch (2^20 x 16 ops,
+// Zipf 0.6: 4.85 -> 4.25 ms) and lost 4 % at Zipf 0.8 (351 -> 367).
+template <int SCHEME>
+constexpr bool CUTS_WAITS = SCHEME != GCC_OCC && SCHEME != GCC_TO && SCHEME != GCC_DET;
 
 // Retry queues.  A transaction that has aborted queue_after times or more and
 // conflicted on a record backs off as above, then takes a ticket in the FIFO
@@ -938,9 +956,6 @@ constexpr uint64_t IDLE_LOOK_NS = 8000, IDLE_TURN_NS = 1000;
 // Admitted transactions always finish their attempt, so a queue never stalls;
 // a transaction still waiting at the kernel deadline gives up and abandons its
 // ticket, and the words are zeroed before every batch.
-// A TicToc transaction joins a queue of at least this many waiting after
-// queue_soon aborts already.
-constexpr int32_t QUEUE_LONG = 8;
 constexpr uint32_t NO_Q = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t queue_of(const ExecArgs& a, uint32_t rec) {
@@ -969,15 +984,17 @@ struct Counters {
 // transaction to be running (a group must never hold an unstarted id that
 // another group waits on while the warp's round waits for that group), so it
 // fetches one id at a time.
-template <unsigned CHUNK>
+// `Id`: 32 bits hold every id and the counter's run past the last one (a batch
+// has at most 2^31 transactions).
+template <unsigned CHUNK, class Id = unsigned long long>
 struct SingleFetch {
     const ExecArgs* a;
-    unsigned long long next_id = 0, end_id = 0;
+    Id next_id = 0, end_id = 0;
     __device__ __forceinline__ bool next(const Lane& L, uint32_t& t, const ExecArgs*& A) {
         if (next_id >= end_id) {
             unsigned long long tt = 0;
             if (L.lig == 0) tt = agg_ticket(&a->st->fetch, CHUNK, &L.n_atom);
-            next_id = __shfl_sync(L.gmask, tt, L.gbase);
+            next_id = __shfl_sync(L.gmask, (Id)tt, L.gbase);
             end_id = next_id + CHUNK;
         }
         if (next_id >= a->n_txns) return false;
@@ -994,14 +1011,7 @@ struct SingleFetch {
 template <int SCHEME, class Work, class Fetch>
 __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, uint64_t deadline,
                            Counters& c) {
-    // OCC's batches end without the wait (an abort there mostly means a commit),
-    // and its contended ones ran 2 % slower with the look.  TO gained 12 % on a
-    // read-mostly batch (2^20 x 16 ops, Zipf 0.6: 4.85 -> 4.25 ms) and lost 2 %
-    // with half writes (27.1 -> 27.7) and 4 % at Zipf 0.8 (351 -> 367), however
-    // seldom it looked: the code alone lengthens each link of the hot chain.
-    // The others gain more (MVCC 3.45 -> 2.30 ms, TicToc and 2PL 10 to 18 %
-    // read-mostly) than they lose at Zipf 0.8 (TicToc 5 %, 2PL 1 %, MVCC 2 %).
-    constexpr bool CUT_WAITS = SCHEME != GCC_OCC && SCHEME != GCC_TO && SCHEME != GCC_DET;
+    constexpr bool CUT_WAITS = CUTS_WAITS<SCHEME>;
     constexpr bool DENSE =
         SCHEME == GCC_NO_WAIT_2PL || SCHEME == GCC_2PL_WAIT_DIE || SCHEME == GCC_DET;
     bool finished = false, has = false, served = false;
@@ -1013,8 +1023,15 @@ __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, 
     uint32_t mv_base = NO_CC;     // MVCC: the transaction's version-store range
     uint64_t first = 0;
     const ExecArgs* A = nullptr;
-    uint64_t look = 0;            // when the warp next looks how many groups are still at work
-    uint32_t cuts = 0, cut_at = 0;   // attempts whose wait was cut short, and the latest of them
+    // CUT_WAITS, in one register each: when the warp next looks how many groups
+    // are still at work (low word of the timer), and of the transaction the
+    // number of attempts whose backoff was cut short (bits 0..4, up to 20) and
+    // the latest of them
+    uint32_t look = CUT_WAITS ? (uint32_t)globaltimer() : 0u, cuts = 0;
+    const uint32_t deadline_64k = (uint32_t)(deadline >> 16);
+    const auto past_deadline = [&](uint64_t now_ns) {
+        return CUT_WAITS ? (int32_t)((uint32_t)(now_ns >> 16) - deadline_64k) > 0 : now_ns > deadline;
+    };
 
     for (;;) {
         // 1. groups without a transaction take the next one
@@ -1069,7 +1086,7 @@ __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, 
                     has = true;
                     attempts = 0;
                     wake = 0;
-                    cuts = cut_at = 0;
+                    cuts = 0;
                     mv_base = NO_CC;
                 }
                 __syncwarp(L.gmask);
@@ -1106,7 +1123,7 @@ __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, 
             const int32_t ahead = (int32_t)(qt - (uint32_t)w);
             if (ahead < (int32_t)a.queue_width) {
                 served = go = true;
-            } else if (now > deadline) {
+            } else if (past_deadline(now)) {
                 expired = true;                // the ticket is abandoned
                 qi = NO_Q;
             } else {
@@ -1156,23 +1173,16 @@ __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, 
                 if (attempts >= a.max_attempts) {
                     if (L.lig == 0) atomicOr(&a.st->error, GCC_DEVERR_ATTEMPTS);
                     outcome = GIVE_UP;
-                } else if (t2 > deadline) {
+                } else if (past_deadline(t2)) {
                     if (L.lig == 0) atomicOr(&a.st->error, GCC_DEVERR_DEADLINE);
                     outcome = GIVE_UP;
                 } else {
                     // randomized backoff first (it breaks the symmetry of two
                     // transactions that keep aborting each other), then the
                     // queue of the record it conflicted on
-                    wake = t2 + backoff_ns(a, t, attempts);
-                    if (a.rq && crec != NO_CC && attempts >= a.queue_after) {
+                    wake = t2 + backoff_ns<SCHEME == GCC_TICTOC || SCHEME == GCC_MVCC>(a, t, attempts);
+                    if (a.rq && crec != NO_CC && attempts >= a.queue_after)
                         pq = queue_of(a, crec);
-                    } else if (SCHEME == GCC_TICTOC && a.rq && crec != NO_CC && attempts >= a.queue_soon) {
-                        // not yet: only a queue that is already long
-                        uint64_t w = 0;
-                        if (L.lig == 0) w = ld_relaxed(a.rq + queue_of(a, crec));
-                        w = __shfl_sync(L.gmask, w, L.gbase);
-                        if ((int32_t)((uint32_t)(w >> 32) - (uint32_t)w) >= QUEUE_LONG) pq = queue_of(a, crec);
-                    }
                 }
             }
             if (outcome == COMMIT) {
@@ -1204,24 +1214,25 @@ __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, 
         // 3. a warp where nobody attempted this round sleeps until its
         // earliest wake-up (32 ns .. 1 us)
         if (!__any_sync(0xffffffffu, go)) {
+            const uint64_t t1 = globaltimer();
             if constexpr (CUT_WAITS) {
-                const uint64_t wnow = __shfl_sync(0xffffffffu, now, 0);     // the same on every lane
-                if (wnow >= look) {
+                const uint32_t wnow = __shfl_sync(0xffffffffu, (uint32_t)t1, 0);     // the same on every lane
+                if ((int32_t)(wnow - look) >= 0) {
                     const uint32_t groups = gridDim.x * (blockDim.x / L.G);
                     const uint32_t busy =
                         groups - __shfl_sync(0xffffffffu, L.lane == 0 ? ld_relaxed_u32(F.idle()) : 0u, 0);
-                    look = wnow + (busy == groups ? 4 * IDLE_LOOK_NS : IDLE_LOOK_NS);
+                    look = wnow + (uint32_t)(busy == groups ? 16 * IDLE_LOOK_NS : IDLE_LOOK_NS);
                     if (has) {
-                        const uint64_t most = (uint64_t)busy * IDLE_TURN_NS << (cuts < 20 ? cuts : 20);
-                        if (wake > wnow + most) {
-                            wake = wnow + mix64(A->seed ^ ((uint64_t)t << 32) ^ attempts) % (most + 1);
-                            if (cut_at != attempts) ++cuts;
-                            cut_at = attempts;
+                        const uint64_t tg = __shfl_sync(L.gmask, t1, L.gbase);
+                        const uint64_t most = (uint64_t)busy * IDLE_TURN_NS << (cuts & 31);
+                        if (wake > tg + most) {
+                            wake = tg + __umul64hi(mix64(A->seed ^ ((uint64_t)t << 32) ^ attempts), most + 1);
+                            if (cuts >> 5 != (attempts & 0x7ffffffu))
+                                cuts = attempts << 5 | ((cuts & 31) < 20 ? (cuts & 31) + 1 : 20);
                         }
                     }
                 }
             }
-            const uint64_t t1 = globaltimer();
             uint32_t rel = 1000;
             if (has && wake > t1) rel = wake - t1 < 1000 ? (uint32_t)(wake - t1) : 1000u;
             else if (has || !finished) rel = 32;   // due now, or about to fetch
@@ -1276,7 +1287,8 @@ __global__ void __launch_bounds__(1024) exec_kernel(const __grid_constant__ Exec
     // one deadline per warp: lanes must agree on every time comparison
     const uint64_t deadline = __shfl_sync(0xffffffffu, globaltimer(), 0) + a.deadline_ns;
     Counters c;
-    SingleFetch<SCHEME == GCC_DET ? 1u : 4u> F{&a};
+    typedef typename std::conditional<CUTS_WAITS<SCHEME>, uint32_t, unsigned long long>::type Id;
+    SingleFetch<SCHEME == GCC_DET ? 1u : 4u, Id> F{&a};
     group_loop<SCHEME, Work>(F, L, S, a.max_ops, deadline, c);
     c.atomics += L.n_atom;
     flush_counters(a.st, c);

@@ -347,7 +347,7 @@ gcc_status enqueue(gcc_multi_plan* pl, cudaStream_t st) {
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
         const uint32_t lanes = pl->p.lanes_per_txn;
-        const uint64_t dl = pl->p.deadline_ns;
+        const uint64_t dl = std::min<uint64_t>(pl->p.deadline_ns, DEADLINE_MAX_NS);
         switch (pl->scheme) {
 #define GCC_MULTI_CASE(SC)                                                                         \
     case SC:                                                                                       \
@@ -516,14 +516,13 @@ gcc_status gcc_multi_plan_create(gcc_scheme scheme, const gcc_multi_batch* b, ui
         a.read_retries = p.read_retries;
         a.inject_ppm = p.inject_abort_ppm;
         a.wait_budget_ns = p.wait_budget_ns;
-        a.deadline_ns = p.deadline_ns;
+        a.deadline_ns = std::min<uint64_t>(p.deadline_ns, gcc::DEADLINE_MAX_NS);
         a.seed = p.seed ^ (0x9E3779B97F4A7C15ull * (i + 1));
         a.rq = (p.retry_queue == 2 || p.immediate_restart) ? nullptr : db->rq;
         a.rq_mask = gcc::RETRY_QUEUES - 1;
         a.queue_turn_ns = p.queue_turn_ns;
         a.queue_width = p.queue_width;
         a.queue_after = queue_after_for(p, scheme);
-        a.queue_soon = queue_soon_for(p, scheme);
         a.seq = db->fold_flags;                  // TicToc: sequence numbers
         a.mv_wts = db->sort.k0;                  // MVCC: the database's version store
         a.mv_next = db->sort.v0;

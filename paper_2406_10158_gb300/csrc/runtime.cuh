@@ -44,7 +44,6 @@ gcc_exec_params defaults();
 gcc_exec_params merged(const gcc_exec_params* in);
 // Aborts before a transaction of `scheme` uses the retry queues.
 uint32_t queue_after_for(const gcc_exec_params& p, gcc_scheme scheme);
-uint32_t queue_soon_for(const gcc_exec_params& p, gcc_scheme scheme);
 gcc_status validate_params(const gcc_exec_params& p);
 gcc_status fail(gcc_status st, const char* fmt, ...);
 // Reset the control words if `scheme` cannot start from their current state.
