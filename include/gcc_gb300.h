@@ -180,7 +180,11 @@ typedef struct gcc_exec_params {
                                   2 = off */
     uint32_t backoff_base_ns;  /* first retry delay, doubled per abort, with
                                   random jitter [128] */
-    uint32_t backoff_cap_ns;   /* largest retry delay [1000000] */
+    uint32_t backoff_cap_ns;   /* largest retry delay [1000000].  With both at
+                                  their defaults 2PL, TicToc and MVCC cut retry
+                                  delays short at a batch's end, when few
+                                  transactions are left to collide with; delays
+                                  set to anything else are kept to */
     uint32_t max_attempts;     /* per transaction, then GCC_TXN_TIMEOUT [2^24] */
     uint32_t read_retries;     /* re-reads of a record seen mid-update before
                                   the attempt aborts [8] */

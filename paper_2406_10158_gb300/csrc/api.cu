@@ -86,6 +86,11 @@ uint32_t queue_after_for(const gcc_exec_params& p, gcc_scheme scheme) {
     return scheme == GCC_OCC ? 64u : scheme == GCC_TICTOC ? 32u : 16u;
 }
 
+uint32_t cut_waits_for(const gcc_exec_params& p) {
+    const gcc_exec_params d = defaults();
+    return p.backoff_base_ns == d.backoff_base_ns && p.backoff_cap_ns == d.backoff_cap_ns;
+}
+
 gcc_exec_params merged(const gcc_exec_params* in) {
     gcc_exec_params p = defaults();
     if (!in) return p;
@@ -399,6 +404,7 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
     a.det_all = p.det_dataflow == 2 ? 1u : 0u;
     a.queue_width = p.queue_width;
     a.queue_after = queue_after_for(p, scheme);
+    a.cut_waits = cut_waits_for(p);
 
     const bool kv = db->d.schema == GCC_SCHEMA_KV;
     // deterministic batches: every record chain by prefix sums (the pipelines

@@ -391,6 +391,7 @@ struct ExecArgs {
     uint32_t queue_turn_ns;     // estimated time per queue turn
     uint32_t queue_width;       // tickets a queue admits at once
     uint32_t queue_after;       // aborts before a transaction uses the queues
+    uint32_t cut_waits;         // backoffs may be cut short at the batch's end
     // MVCC version store of the batch: entry i = (wts, next, record, field,
     // value); capacity n_ops (one entry per committed write)
     uint32_t* mv_wts;

@@ -928,9 +928,10 @@ __device__ __forceinline__ uint64_t backoff_ns(const ExecArgs& a, uint32_t t, ui
 // turn each.  Long transactions that all conflict need more, so the bound
 // doubles with every attempt of a transaction that was cut short and aborted
 // again, back to the full windows (a fixed bound livelocked 60-op transactions
-// on 512 records).  Read-mostly MVCC batch of 2^18 transactions, Zipf 0.6:
-// 3.54 ms without, 2.27 with (2.80 at 4 us a group); looking every 2 us
-// instead of 8 slowed contended batches by 3 %.
+// on 512 records).  Windows the caller set are not cut (ExecArgs::cut_waits),
+// nor are waits in a retry queue.  Read-mostly MVCC batch of 2^18 transactions,
+// Zipf 0.6: 3.54 ms without, 2.27 with (2.80 at 4 us a group); looking every
+// 2 us instead of 8 slowed contended batches by 3 %.
 // The look's state takes two registers, the transaction counter and the deadline
 // one each instead of two, because every register it takes from the attempts
 // lengthens each link of a hot record's chain: with six for the look TicToc
@@ -1222,7 +1223,7 @@ __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, 
                     const uint32_t busy =
                         groups - __shfl_sync(0xffffffffu, L.lane == 0 ? ld_relaxed_u32(F.idle()) : 0u, 0);
                     look = wnow + (uint32_t)(busy == groups ? 16 * IDLE_LOOK_NS : IDLE_LOOK_NS);
-                    if (has) {
+                    if (has && qi == NO_Q && A->cut_waits) {
                         const uint64_t tg = __shfl_sync(L.gmask, t1, L.gbase);
                         const uint64_t most = (uint64_t)busy * IDLE_TURN_NS << (cuts & 31);
                         if (wake > tg + most) {

@@ -523,6 +523,7 @@ gcc_status gcc_multi_plan_create(gcc_scheme scheme, const gcc_multi_batch* b, ui
         a.queue_turn_ns = p.queue_turn_ns;
         a.queue_width = p.queue_width;
         a.queue_after = queue_after_for(p, scheme);
+        a.cut_waits = cut_waits_for(p);
         a.seq = db->fold_flags;                  // TicToc: sequence numbers
         a.mv_wts = db->sort.k0;                  // MVCC: the database's version store
         a.mv_next = db->sort.v0;

@@ -44,6 +44,8 @@ gcc_exec_params defaults();
 gcc_exec_params merged(const gcc_exec_params* in);
 // Aborts before a transaction of `scheme` uses the retry queues.
 uint32_t queue_after_for(const gcc_exec_params& p, gcc_scheme scheme);
+// Whether backoffs may be cut short at a batch's end: other than the default ones are the caller's.
+uint32_t cut_waits_for(const gcc_exec_params& p);
 gcc_status validate_params(const gcc_exec_params& p);
 gcc_status fail(gcc_status st, const char* fmt, ...);
 // Reset the control words if `scheme` cannot start from their current state.

@@ -58,3 +58,22 @@ def test_small_batches_of_every_launch_shape_end(eng, scheme):
             assert stats["committed"] == 333, (lanes, warps, stats)
             rep = oracle.replay_check(table, db.read_kv(), batch, res, reads)
             assert rep["ok"], (lanes, warps, rep)
+
+
+@pytest.mark.parametrize("scheme", SCHEMES)
+def test_backoff_the_caller_set_is_kept(eng, scheme):
+    """256 transactions on one record, delays of 0, 20 or 40 ms: each delay is
+    sat out in full, so the kernel takes at least the 20 ms of the shortest one
+    that is not zero (one microsecond per lane group would be 0.26 ms)."""
+    table = wl.kv_table_splitmix(35, 16, 1)
+    batch = wl.kv_batch_from_lists([[(3, 0, 1, t + 1, 0)] for t in range(256)])
+    with eng.Database("kv", n_records=16, n_fields=1, field_bytes=8, max_batch_txns=256) as db:
+        db.load_kv(table)
+        res, reads, stats = db.run(scheme, batch, eng.params(
+            backoff_base_ns=20_000_000, backoff_cap_ns=40_000_000, retry_queue=2))
+        final = db.read_kv()
+    assert stats["committed"] == 256, stats
+    assert oracle.replay_check(table, final, batch, res, reads)["ok"]
+    waited = res["attempts"][res["attempts"] > 1].size
+    assert waited >= 32, stats                      # all of them draw zero: below 2^-32
+    assert stats["kernel_ms"] >= 20.0, stats
