@@ -444,12 +444,9 @@ oe_in_order(const __grid_constant__ ExecArgs a, const __grid_constant__ OeTables
         }
         for (uint32_t p = at; p < end + 1; p += 32) {
             const uint32_t m = end - p + 1 < 32 ? end - p + 1 : 32;
-            uint64_t op = 0;
             __syncwarp();
-            if (lane < (int)m) {
-                op = f.op(op0, sv[p + lane]);
-                s_o[wib][lane] = a.operands[op];
-            }
+            const uint64_t op = lane < (int)m ? f.op(op0, sv[p + lane]) : ~0ull;
+            if (lane < (int)m) s_o[wib][lane] = op < a.n_ops ? a.operands[op] : make_ulonglong2(0ull, 0ull);
             __syncwarp();
             if (lane == 0)
                 for (uint32_t i = 0; i < m; ++i) {
@@ -462,7 +459,7 @@ oe_in_order(const __grid_constant__ ExecArgs a, const __grid_constant__ OeTables
                     rem += o.y;
                 }
             __syncwarp();
-            if (lane < (int)m) a.reads[op] = s_r[wib][lane];
+            if (op < a.n_ops) a.reads[op] = s_r[wib][lane];
         }
         if (lane == 0) {
             T.c[S_QUANTITY][row] = q;

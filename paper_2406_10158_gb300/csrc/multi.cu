@@ -183,7 +183,9 @@ __global__ void multi_rank_keys(const ExecArgs* __restrict__ args, const uint32_
 __global__ void multi_batch_keys(const uint32_t* __restrict__ prefix, uint32_t n, uint64_t total,
                                  uint32_t* __restrict__ keys, const uint32_t* __restrict__ vals) {
     const uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < total) keys[p] = find_batch(prefix, n, vals[p]);
+    if (p >= total) return;
+    const uint32_t g = vals[p];
+    keys[p] = g < total ? find_batch(prefix, n, g) : n - 1;    // past the end: a sort that gave up
 }
 
 __global__ void multi_ranks(const ExecArgs* __restrict__ args, const uint32_t* __restrict__ prefix,
@@ -191,6 +193,7 @@ __global__ void multi_ranks(const ExecArgs* __restrict__ args, const uint32_t* _
     const uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= total) return;
     const uint32_t g = vals[p];
+    if (g >= total) return;                      // a sort that gave up
     const uint32_t i = find_batch(prefix, n, g);
     const ExecArgs& a = args[i];
     const uint32_t t = g - prefix[i];
@@ -241,13 +244,15 @@ __global__ void multi_tt_keys(const ExecArgs* __restrict__ args, const uint32_t*
     const uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= total) return;
     const uint32_t g = pass == 0 ? (uint32_t)p : vals[p];
-    const uint32_t i = find_batch(prefix, n, g);
-    const ExecArgs& a = args[i];
-    const uint32_t t = g - prefix[i];
     uint32_t k = 0xffffffffu;
-    if (a.results[t].status == GCC_TXN_COMMITTED)
-        k = pass == 0 ? a.seq[t] : pass == 1 ? (uint32_t)a.order_key[t]
-                                             : (uint32_t)(a.order_key[t] >> 32);
+    if (g < total) {                             // else a sort that gave up
+        const uint32_t i = find_batch(prefix, n, g);
+        const ExecArgs& a = args[i];
+        const uint32_t t = g - prefix[i];
+        if (a.results[t].status == GCC_TXN_COMMITTED)
+            k = pass == 0 ? a.seq[t] : pass == 1 ? (uint32_t)a.order_key[t]
+                                                 : (uint32_t)(a.order_key[t] >> 32);
+    }
     keys[p] = k;
     vals[p] = g;
 }

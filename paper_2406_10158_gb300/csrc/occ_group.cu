@@ -63,6 +63,7 @@ __global__ void unit_links(const uint32_t* __restrict__ sk, const uint32_t* __re
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const uint32_t k = sk[p], t = sv[p];
+    if (t >= n) return;                          // a sort that gave up
     if (k == none_key) { link[t] = UNIT_NONE; return; }
     uint32_t lo = 0, hi = p;                     // first position of key k
     while (lo < hi) {

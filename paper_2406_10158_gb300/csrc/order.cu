@@ -69,8 +69,11 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* w
 // of twice and needs one launch instead of three.
 //
 // Tiles are numbered by a ticket, so a tile's predecessors are always running
-// or done and the wait ends; it is bounded all the same (SPIN_MAX), and a
-// tile that gave up sets GCC_DEVERR_WAIT_BUDGET and stays in bounds.
+// or done and the wait ends; it is bounded all the same (SPIN_MAX).  A tile
+// that gave up sets GCC_DEVERR_WAIT_BUDGET and scatters in bounds, but its
+// output positions overlap others': what they leave out holds words of an
+// earlier use of the buffer, so whoever reads a sorted pair checks it against
+// the array it indexes.
 template <class W> struct Count {
     static constexpr int BITS = sizeof(W) * 8 - 2;
     static constexpr W OWN = W(1) << BITS, UP_TO = W(2) << BITS, MASK = (W(1) << BITS) - 1;
@@ -361,7 +364,8 @@ __global__ void det_flags(const uint64_t* __restrict__ ops, const uint32_t* __re
                           uint64_t n, uint32_t* __restrict__ flags) {
     const uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
-    flags[p] = kind_writes((uint32_t)(ops[sv[p]] >> 40) & 0xffu) ? 1u : 0u;
+    const uint32_t op = sv[p];
+    flags[p] = op < n && kind_writes((uint32_t)(ops[op] >> 40) & 0xffu) ? 1u : 0u;
 }
 
 // need: a write (or, when every access conflicts, any op) waits for all
@@ -373,8 +377,8 @@ __global__ void det_need(const uint64_t* __restrict__ ops, const uint32_t* __res
     const uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const uint32_t key = sk[p];
-    if (key == none) return;
     const uint32_t op = sv[p];
+    if (key >= none || op >= n) return;
     const bool w = kind_writes((uint32_t)(ops[op] >> 40) & 0xffu);
     need[op] = (w || all_conflict) ? (uint32_t)p : wpre[p];
     if (p == 0 || sk[p - 1] != key) meta[key] = ((uint64_t)p << 32) | wpre[p];
@@ -523,7 +527,7 @@ rank_assign(const __grid_constant__ ExecArgs a, const RankScratch r, int scheme)
 __global__ void dense_rank(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv,
                            uint32_t n, gcc_txn_result* __restrict__ res) {
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n || sk[p] == 0xffffffffu) return;
+    if (p >= n || sk[p] == 0xffffffffu || sv[p] >= n) return;
     res[sv[p]].commit_order = p;
 }
 
@@ -540,7 +544,7 @@ __global__ void tt_emit(const gcc_txn_result* __restrict__ res,
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const uint32_t t = pass == 0 ? p : sv[p];
-    const bool c = res[t].status == GCC_TXN_COMMITTED;
+    const bool c = t < n && res[t].status == GCC_TXN_COMMITTED;
     uint32_t k = 0xffffffffu;
     if (c) k = pass == 0 ? seq[t] : pass == 1 ? (uint32_t)okey[t] : (uint32_t)(okey[t] >> 32);
     keys[p] = k;

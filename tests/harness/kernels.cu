@@ -1,0 +1,92 @@
+// kernels.cu -- entry points for tests into kernels that the library only
+// launches itself.  One translation unit of the engine is included per PART, so
+// that its internal kernels can be called with buffers of the test's own.
+#include <cuda_runtime.h>
+
+#if PART == 0
+#include "order.cu"
+#elif PART == 1
+#include "occ_group.cu"
+#elif PART == 2
+#include "multi.cu"
+#elif PART == 3
+#include "det_oe.cu"
+#endif
+
+namespace {
+unsigned grid_of(uint64_t n) { return (unsigned)((n + 255) / 256); }
+int done() {
+    const cudaError_t e = cudaGetLastError();
+    return (int)(e != cudaSuccess ? e : cudaDeviceSynchronize());
+}
+}  // namespace
+
+extern "C" {
+#if PART == 0
+int h_dense_rank(const uint32_t* sk, const uint32_t* sv, uint32_t n, gcc_txn_result* res) {
+    gcc::dense_rank<<<grid_of(n), 256>>>(sk, sv, n, res);
+    return done();
+}
+int h_tt_emit(const gcc_txn_result* res, const unsigned long long* okey, const uint32_t* seq, const uint32_t* sv,
+              int pass, uint32_t n, uint32_t* keys, uint32_t* vals) {
+    gcc::tt_emit<<<grid_of(n), 256>>>(res, okey, seq, sv, pass, n, keys, vals);
+    return done();
+}
+int h_det_flags(const uint64_t* ops, const uint32_t* sv, uint64_t n, uint32_t* flags) {
+    gcc::det_flags<<<grid_of(n), 256>>>(ops, sv, n, flags);
+    return done();
+}
+int h_det_need(const uint64_t* ops, const uint32_t* sk, const uint32_t* sv, const uint32_t* wpre, uint64_t n,
+               uint32_t none, uint32_t* need, uint64_t* meta) {
+    gcc::det_need<<<grid_of(n), 256>>>(ops, sk, sv, wpre, n, none, 0, need, meta);
+    return done();
+}
+#elif PART == 1
+int h_unit_links(const uint32_t* sk, const uint32_t* sv, uint32_t n, uint32_t U, uint32_t none, uint32_t* link) {
+    gcc::unit_links<<<grid_of(n), 256>>>(sk, sv, n, U, none, link);
+    return done();
+}
+#elif PART == 2
+// Two databases' results and commit keys; `prefix` on the device.
+int h_multi(gcc_txn_result* r0, gcc_txn_result* r1, unsigned long long* o0, unsigned long long* o1, uint32_t* s0,
+            uint32_t* s1, const uint32_t* prefix, uint64_t total, uint32_t* batch_keys, uint32_t* tt_keys,
+            uint32_t* vals) {
+    gcc::ExecArgs a[2]{}, *d = nullptr;
+    a[0].results = r0;
+    a[1].results = r1;
+    a[0].order_key = o0;
+    a[1].order_key = o1;
+    a[0].seq = s0;
+    a[1].seq = s1;
+    cudaError_t e = cudaMalloc(&d, sizeof a);
+    if (e == cudaSuccess) e = cudaMemcpy(d, a, sizeof a, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return (int)e;
+    gcc::multi_batch_keys<<<grid_of(total), 256>>>(prefix, 2, total, batch_keys, vals);
+    gcc::multi_tt_keys<<<grid_of(total), 256>>>(d, prefix, 2, total, 2, tt_keys, vals);
+    gcc::multi_ranks<<<grid_of(total), 256>>>(d, prefix, 2, total, vals);
+    const int r = done();
+    cudaFree(d);
+    return r;
+}
+#elif PART == 3
+// A run of stock accesses in positions 0..n-1 (one warehouse).
+int h_in_order(uint64_t* quantity, uint64_t* ytd, uint64_t* cnt, uint64_t* remote, const uint32_t* sk,
+               const uint32_t* sv, uint32_t n, const ulonglong2* operands, ulonglong2* reads, uint64_t n_ops,
+               const uint32_t* n_odd, const uint32_t* odd) {
+    gcc::ExecArgs a{};
+    a.n_warehouses = 1;
+    a.n_meta = 130011;
+    a.operands = operands;
+    a.reads = reads;
+    a.n_ops = n_ops;
+    gcc::OeTables T{};
+    T.c[gcc::oe::S_QUANTITY] = quantity;
+    T.c[gcc::oe::S_YTD] = ytd;
+    T.c[gcc::oe::S_ORDER_CNT] = cnt;
+    T.c[gcc::oe::S_REMOTE_CNT] = remote;
+    const gcc::AccessKeys f = gcc::access_keys(a.n_meta, n, gcc::OE_CHUNK_LOG2, gcc::OE_SORT_LOG2, true);
+    gcc::oe_in_order<<<1, 256>>>(a, T, f, sk, sv, 0, 0, n, n_odd, odd);
+    return done();
+}
+#endif
+}
