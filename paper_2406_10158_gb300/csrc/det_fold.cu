@@ -76,7 +76,7 @@ __device__ __forceinline__ Sum sum_add(Sum a, Sum b) { return Sum{a.lo + b.lo, (
 // latency better than 3 (6,573 against 6,795; 5 spill, 6,606).
 template <int G>
 __global__ void __launch_bounds__(256, G == 32 ? 4 : 1)
-fold_validate(const __grid_constant__ ExecArgs a, const AccessKeys f, uint32_t* __restrict__ keys,
+fold_validate(const __grid_constant__ ExecArgs a, const AccessKeys f, uint32_t* keys,
               uint32_t* work, uint32_t per_block) {
     constexpr int GROUPS = 256 / G, U = G == 32 ? 2 : 4;
     __shared__ DigitHist h[SORT_MAX_PASSES];
@@ -251,8 +251,8 @@ __device__ __forceinline__ Sum fold_look_back(const ulonglong2* desc, int64_t ti
 // eight launches of this one 0.83 ms.
 template <int FB>
 __global__ void __launch_bounds__(FT_THREADS, 4)
-fold_tiles(const __grid_constant__ ExecArgs a, const AccessKeys f, const uint32_t* __restrict__ sk,
-           const uint32_t* __restrict__ sv, uint64_t op0, uint32_t c0, uint32_t c1,
+fold_tiles(const __grid_constant__ ExecArgs a, const AccessKeys f, const uint32_t* sk,
+           const uint32_t* sv, uint64_t op0, uint32_t c0, uint32_t c1,
            uint32_t* ticket, ulonglong2* desc) {
     constexpr int ITEMS = FT_ITEMS<FB>;
     __shared__ uint32_t s_tile;

@@ -57,7 +57,7 @@ constexpr int64_t Q_LO = 10, Q_HI = 100, Q_MOD = 91;
 // 2^18 transactions (a warp per transaction and all pairs: 226 us).
 __global__ void __launch_bounds__(256)
 oe_validate(const __grid_constant__ ExecArgs a, const __grid_constant__ OeTables T, const AccessKeys f,
-            uint32_t* __restrict__ keys, uint32_t* work, uint32_t per_block) {
+            uint32_t* keys, uint32_t* work, uint32_t per_block) {
     constexpr int U = 2, STEP = 16 * U;
     __shared__ DigitHist h[SORT_MAX_PASSES];
     const int lane = threadIdx.x & 31, lig = lane & 15;
@@ -299,7 +299,7 @@ __device__ __forceinline__ void store_record(const OeTables& T, const Access& x,
 // its accesses read.
 __global__ void __launch_bounds__(OF_THREADS)
 oe_fold(const __grid_constant__ ExecArgs a, const __grid_constant__ OeTables T, const AccessKeys f,
-        const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint64_t op0, uint32_t c0,
+        const uint32_t* sk, const uint32_t* sv, uint64_t op0, uint32_t c0,
         uint32_t c1, uint32_t* ticket, ulonglong2* desc, uint32_t* n_odd, uint32_t* odd) {
     __shared__ uint32_t s_tile;
     __shared__ Add s_tot[OF_WARPS];
@@ -416,7 +416,7 @@ oe_fold(const __grid_constant__ ExecArgs a, const __grid_constant__ OeTables T, 
 // lane 0 applies the quantity rule op by op, 32 staged at a time.
 __global__ void __launch_bounds__(256)
 oe_in_order(const __grid_constant__ ExecArgs a, const __grid_constant__ OeTables T, const AccessKeys f,
-            const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint64_t op0, uint32_t c0,
+            const uint32_t* sk, const uint32_t* sv, uint64_t op0, uint32_t c0,
             uint32_t c1, const uint32_t* n_odd, const uint32_t* odd) {
     __shared__ ulonglong2 s_o[8][32], s_r[8][32];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;

@@ -322,7 +322,10 @@ __host__ __device__ __forceinline__ uint32_t cc_record(uint64_t d, int schema, u
 // in the stream drains; it calls after_previous() before it touches memory,
 // which waits until the predecessor has completed and its writes are visible,
 // and lets its own successor be scheduled in turn.  A chain of short kernels
-// then costs little more than its kernels.
+// then costs little more than its kernels.  Such a kernel may be resident while
+// its predecessor still writes, so none of its pointers is __restrict__: const
+// and restrict together promise data that nobody writes during the kernel, and
+// let a load move above the wait.
 __device__ __forceinline__ void after_previous() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -120,8 +120,8 @@ __device__ __forceinline__ W look_back(const W* desc, int64_t tile, int t, unsig
 
 // Histograms of every pass's digits.
 __global__ void __launch_bounds__(RS_BLOCK)
-rs_hist(const uint32_t* __restrict__ keys, size_t n, int bits, int passes, int digit_bits,
-        uint32_t* __restrict__ hist) {
+rs_hist(const uint32_t* keys, size_t n, int bits, int passes, int digit_bits,
+        uint32_t* hist) {
     __shared__ uint32_t h[SORT_MAX_PASSES][256];
     after_previous();
     for (int p = 0; p < SORT_MAX_PASSES; ++p) h[p][threadIdx.x] = 0;
@@ -166,9 +166,9 @@ rs_hist(const uint32_t* __restrict__ keys, size_t n, int bits, int passes, int d
 // of the key moves to bit 31 of the value.
 template <class W, int ITEMS>
 __global__ void __launch_bounds__(RS_BLOCK)
-rs_pass(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin,
-        uint32_t* __restrict__ kout, uint32_t* __restrict__ vout, size_t n, int shift, int width,
-        int flagged, const uint32_t* __restrict__ hist, W* desc, W* desc_next, uint32_t* ticket,
+rs_pass(const uint32_t* kin, const uint32_t* vin,
+        uint32_t* kout, uint32_t* vout, size_t n, int shift, int width,
+        int flagged, const uint32_t* hist, W* desc, W* desc_next, uint32_t* ticket,
         unsigned* err) {
     constexpr int TILE = RS_BLOCK * ITEMS;
     __shared__ uint32_t gbase[256];            // global start of each digit's run, less dstart
