@@ -218,6 +218,51 @@ __device__ __forceinline__ void flush_digits(const AccessKeys& f, DigitHist* h, 
     }
 }
 
+// --- sums across tiles --------------------------------------------------------
+// A tile of sorted accesses publishes one 16-byte descriptor: its sum S and in
+// bits 62..63 of the second word its state.  TAIL: no slot's accesses begin in
+// the tile, the sum is the whole tile's and what comes before adds to it.
+// WHOLE: the sum from the beginning of the slot whose accesses run on past the
+// tile.
+constexpr uint64_t TAIL = 1ull << 62, WHOLE = 2ull << 62;
+
+// The sum of the accesses before `tile` to the slot that runs into it, by the
+// lanes of one warp, 32 predecessors at a time (usually one: nearly every tile
+// begins some slot).  Acquire loads: the caller may write that slot only after
+// every tile it runs through has read its initial value.  Every lane's acquires
+// come before whatever any lane of the warp does next -- lane 0 publishes the
+// tile's own WHOLE, which a later tile takes as word of all tiles before --
+// and shuffles order no memory, so the warp meets at a barrier at the end.
+template <class S>
+__device__ __forceinline__ S look_back(const ulonglong2* desc, int64_t tile, unsigned* err) {
+    const int lane = threadIdx.x & 31;
+    S sum{};
+    uint32_t spins = 0;
+    for (int64_t p = tile - 1; p >= 0;) {
+        ulonglong2 w = make_ulonglong2(0ull, WHOLE);
+        if (p - lane >= 0) w = ld128_acquire(desc + (p - lane));
+        const unsigned whole = __ballot_sync(0xffffffffu, w.y >= WHOLE);
+        const unsigned none = __ballot_sync(0xffffffffu, w.y == 0);
+        const int upto = whole ? __ffs(whole) - 1 : 31;             // last lane that counts
+        const unsigned need = upto == 31 ? 0xffffffffu : (2u << upto) - 1u;
+        if (none & need) {
+            if (++spins > DET_SPIN_MAX) {
+                if (lane == 0) atomicOr(err, GCC_DEVERR_WAIT_BUDGET);
+                break;
+            }
+            continue;
+        }
+        S x = lane <= upto ? S::unpack(w) : S{};
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x = x + x.of_lane_xor(o);
+        sum = sum + x;
+        if (whole) break;
+        p -= 32;
+    }
+    __syncwarp();
+    return sum;
+}
+
 // Ends a batch: counts the commits.  The validation pass gave every valid
 // transaction its id as its commit order, which is right when every
 // transaction is valid; otherwise the order is the rank among the valid ones,

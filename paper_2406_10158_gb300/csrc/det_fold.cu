@@ -57,8 +57,14 @@ __device__ __forceinline__ uint32_t d_kind(uint64_t d) { return (uint32_t)(d >> 
 struct Sum {
     uint64_t lo;
     uint32_t hi;           // modulo 2^16
+    // as a tile descriptor: x lane 0, y bits 0..15 bytes 8-9 (and the state)
+    __device__ __forceinline__ ulonglong2 pack(uint64_t state) const { return make_ulonglong2(lo, hi | state); }
+    static __device__ __forceinline__ Sum unpack(ulonglong2 w) { return Sum{w.x, (uint32_t)w.y & 0xFFFFu}; }
+    __device__ __forceinline__ Sum of_lane_xor(int o) const {
+        return Sum{__shfl_xor_sync(0xffffffffu, lo, o), __shfl_xor_sync(0xffffffffu, hi, o)};
+    }
 };
-__device__ __forceinline__ Sum sum_add(Sum a, Sum b) { return Sum{a.lo + b.lo, (a.hi + b.hi) & 0xFFFFu}; }
+__device__ __forceinline__ Sum operator+(Sum a, Sum b) { return Sum{a.lo + b.lo, (a.hi + b.hi) & 0xFFFFu}; }
 
 // --- validation and access table ---------------------------------------------
 // A lane group of G lanes per transaction (G the smallest of 8, 16, 32 that
@@ -195,48 +201,6 @@ __device__ __forceinline__ ulonglong2 slot_plus(ulonglong2 v, Sum s) {
     return make_ulonglong2(v.x + s.lo, 0ull);
 }
 
-// Tile descriptor: x the sum's lane 0, y bits 0..15 its bytes 8-9, bits 62..63
-// the state.  TAIL: no slot's accesses begin in the tile, the sum is the whole
-// tile's and what comes before adds to it.  WHOLE: the sum from the beginning
-// of the slot whose accesses run on past the tile.
-constexpr uint64_t TAIL = 1ull << 62, WHOLE = 2ull << 62;
-
-// The sum of the accesses before `tile` to the slot that runs into it, by the
-// lanes of one warp, 32 predecessors at a time (usually one: nearly every tile
-// begins some slot).  Acquire loads: the caller may write that slot only after
-// every tile it runs through has read its initial value.
-__device__ __forceinline__ Sum fold_look_back(const ulonglong2* desc, int64_t tile, unsigned* err) {
-    const int lane = threadIdx.x & 31;
-    Sum sum{0, 0};
-    uint32_t spins = 0;
-    for (int64_t p = tile - 1; p >= 0;) {
-        ulonglong2 w = make_ulonglong2(0ull, WHOLE);
-        if (p - lane >= 0) w = ld128_acquire(desc + (p - lane));
-        const unsigned whole = __ballot_sync(0xffffffffu, w.y >= WHOLE);
-        const unsigned none = __ballot_sync(0xffffffffu, w.y == 0);
-        const int upto = whole ? __ffs(whole) - 1 : 31;             // last lane that counts
-        const unsigned need = upto == 31 ? 0xffffffffu : (2u << upto) - 1u;
-        if (none & need) {
-            if (++spins > DET_SPIN_MAX) {
-                if (lane == 0) atomicOr(err, GCC_DEVERR_WAIT_BUDGET);
-                return sum;
-            }
-            continue;
-        }
-        uint64_t lo = lane <= upto ? w.x : 0ull;
-        uint32_t hi = lane <= upto ? (uint32_t)w.y & 0xFFFFu : 0u;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            lo += __shfl_xor_sync(0xffffffffu, lo, o);
-            hi += __shfl_xor_sync(0xffffffffu, hi, o);
-        }
-        sum = sum_add(sum, Sum{lo, hi});
-        if (whole) break;
-        p -= 32;
-    }
-    return sum;
-}
-
 // One tile of sorted accesses: an access reads its slot's initial value
 // plus the sum of the deltas before it, the last access of a slot stores the
 // final value.  Within the tile every initial value is read before the block
@@ -315,7 +279,7 @@ fold_tiles(const __grid_constant__ ExecArgs a, const AccessKeys f, const uint32_
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
         if (head >> i & 1) run = Sum{0, 0};
-        run = sum_add(run, dl[i]);
+        run = run + dl[i];
         seen ^= (uint32_t)init[i].x;
     }
     // within the warp: inclusive sums since the last lane that begins a slot
@@ -327,7 +291,7 @@ fold_tiles(const __grid_constant__ ExecArgs a, const AccessKeys f, const uint32_
     for (int o = 1; o < 32; o <<= 1) {
         const uint64_t lo = __shfl_up_sync(0xffffffffu, inc.lo, o);
         const uint32_t hi = FB == 16 ? __shfl_up_sync(0xffffffffu, inc.hi, o) : 0u;
-        if (lane - o >= start) inc = sum_add(inc, Sum{lo, hi});
+        if (lane - o >= start) inc = inc + Sum{lo, hi};
     }
     Sum carry;                                 // what precedes the thread, in the warp
     carry.lo = __shfl_up_sync(0xffffffffu, inc.lo, 1);
@@ -347,17 +311,14 @@ fold_tiles(const __grid_constant__ ExecArgs a, const AccessKeys f, const uint32_
 #pragma unroll
         for (int w = 0; w < FT_WARPS; ++w) {
             if (s_hi[w] >> 31) { tot = Sum{0, 0}; begins = true; }
-            tot = sum_add(tot, Sum{s_lo[w], s_hi[w] & 0xFFFFu});
+            tot = tot + Sum{s_lo[w], s_hi[w] & 0xFFFFu};
         }
         const bool whole = begins || tile == 0;
-        if (lane == 0) st128_release(desc + tile, make_ulonglong2(tot.lo, tot.hi | (whole ? WHOLE : TAIL)));
+        if (lane == 0) st128_release(desc + tile, tot.pack(whole ? WHOLE : TAIL));
         Sum before{0, 0};
         if (__shfl_sync(0xffffffffu, runs_in, 0)) {
-            before = fold_look_back(desc, tile, &a.st->error);
-            if (!whole && lane == 0) {
-                const Sum all = sum_add(before, tot);
-                st128_release(desc + tile, make_ulonglong2(all.lo, all.hi | WHOLE));
-            }
+            before = look_back<Sum>(desc, tile, &a.st->error);
+            if (!whole && lane == 0) st128_release(desc + tile, (before + tot).pack(WHOLE));
         }
         if (lane == 0) s_carry = before;
     }
@@ -365,17 +326,17 @@ fold_tiles(const __grid_constant__ ExecArgs a, const AccessKeys f, const uint32_
     if (!(heads & (0xffffffffu >> (31 - lane)) & ~(1u << lane))) {   // no lane before begins a slot
         bool open = true;
         for (int w = warp - 1; w >= 0 && open; --w) {
-            carry = sum_add(carry, Sum{s_lo[w], s_hi[w] & 0xFFFFu});
+            carry = carry + Sum{s_lo[w], s_hi[w] & 0xFFFFu};
             open = !(s_hi[w] >> 31);
         }
-        if (open) carry = sum_add(carry, s_carry);
+        if (open) carry = carry + s_carry;
     }
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
         if (head >> i & 1) carry = Sum{0, 0};
         if (!(live >> i & 1)) continue;
         a.reads[f.op(op0, v[i])] = slot_plus<FB>(init[i], carry);
-        carry = sum_add(carry, dl[i]);
+        carry = carry + dl[i];
         const bool last = base + i + 1 >= c1 || (i + 1 < ITEMS ? k[(i + 1) % ITEMS] : next) != k[i];
         if (last && (carry.lo | carry.hi)) {                     // unchanged slots are not stored
             const ulonglong2 fin = slot_plus<FB>(init[i], carry);

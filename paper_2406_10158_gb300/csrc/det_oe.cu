@@ -168,59 +168,30 @@ oe_validate(const __grid_constant__ ExecArgs a, const __grid_constant__ OeTables
 // What a run of accesses adds to its record: amount (Payment amounts, order
 // quantities), count (orders, payments), remote lines; ODD in `r` marks a
 // stock run outside the regular ranges.
+constexpr uint32_t ODD = 0x80000000u;
 struct Add {
     uint64_t a;
     uint32_t n, r;
+    // as a tile descriptor: x the amount, y bits 0..29 the count, 30..59 the
+    // remote lines, 60 ODD (and the state)
+    __device__ __forceinline__ ulonglong2 pack(uint64_t state) const {
+        return make_ulonglong2(a, (uint64_t)n | (uint64_t)(r & ~ODD) << 30 | (r & ODD ? 1ull << 60 : 0ull) | state);
+    }
+    static __device__ __forceinline__ Add unpack(ulonglong2 w) {
+        return Add{w.x, (uint32_t)w.y & 0x3fffffffu,
+                   ((uint32_t)(w.y >> 30) & 0x3fffffffu) | (w.y >> 60 & 1 ? ODD : 0u)};
+    }
+    __device__ __forceinline__ Add of_lane_xor(int o) const {
+        return Add{__shfl_xor_sync(0xffffffffu, a, o), __shfl_xor_sync(0xffffffffu, n, o),
+                   __shfl_xor_sync(0xffffffffu, r, o)};
+    }
 };
-constexpr uint32_t ODD = 0x80000000u;
 __device__ __forceinline__ Add operator+(Add x, Add y) {
     return Add{x.a + y.a, x.n + y.n, ((x.r + y.r) & ~ODD) | ((x.r | y.r) & ODD)};
-}
-// Tile descriptor: x the amount, y bits 0..29 the count, 30..59 the remote
-// lines, 60 ODD, 62..63 the state (as in det_fold.cu).
-constexpr uint64_t TAIL = 1ull << 62, WHOLE = 2ull << 62;
-__device__ __forceinline__ ulonglong2 pack(Add s, uint64_t state) {
-    return make_ulonglong2(s.a, (uint64_t)s.n | (uint64_t)(s.r & ~ODD) << 30 |
-                                    (s.r & ODD ? 1ull << 60 : 0ull) | state);
-}
-__device__ __forceinline__ Add unpack(ulonglong2 w) {
-    return Add{w.x, (uint32_t)w.y & 0x3fffffffu,
-               ((uint32_t)(w.y >> 30) & 0x3fffffffu) | (w.y >> 60 & 1 ? ODD : 0u)};
 }
 __device__ __forceinline__ Add shfl_up(Add s, int o) {
     return Add{__shfl_up_sync(0xffffffffu, s.a, o), __shfl_up_sync(0xffffffffu, s.n, o),
                __shfl_up_sync(0xffffffffu, s.r, o)};
-}
-
-// As det_fold.cu's: what precedes `tile` on the record that runs into it.
-__device__ __forceinline__ Add oe_look_back(const ulonglong2* desc, int64_t tile, unsigned* err) {
-    const int lane = threadIdx.x & 31;
-    Add sum{0, 0, 0};
-    uint32_t spins = 0;
-    for (int64_t p = tile - 1; p >= 0;) {
-        ulonglong2 w = make_ulonglong2(0ull, WHOLE);
-        if (p - lane >= 0) w = ld128_acquire(desc + (p - lane));
-        const unsigned whole = __ballot_sync(0xffffffffu, w.y >= WHOLE);
-        const unsigned none = __ballot_sync(0xffffffffu, w.y == 0);
-        const int upto = whole ? __ffs(whole) - 1 : 31;             // last lane that counts
-        const unsigned need = upto == 31 ? 0xffffffffu : (2u << upto) - 1u;
-        if (none & need) {
-            if (++spins > DET_SPIN_MAX) {
-                if (lane == 0) atomicOr(err, GCC_DEVERR_WAIT_BUDGET);
-                return sum;
-            }
-            continue;
-        }
-        Add x = lane <= upto ? unpack(w) : Add{0, 0, 0};
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            x = x + Add{__shfl_xor_sync(0xffffffffu, x.a, o), __shfl_xor_sync(0xffffffffu, x.n, o),
-                        __shfl_xor_sync(0xffffffffu, x.r, o)};
-        sum = sum + x;
-        if (whole) break;
-        p -= 32;
-    }
-    return sum;
 }
 
 enum Class { WAREHOUSE, DISTRICT, CUSTOMER, STOCK };
@@ -382,11 +353,11 @@ oe_fold(const __grid_constant__ ExecArgs a, const __grid_constant__ OeTables T, 
             tot = tot + s_tot[w];
         }
         const bool whole = begins || tile == 0;
-        if (lane == 0) st128_release(desc + tile, pack(tot, whole ? WHOLE : TAIL));
+        if (lane == 0) st128_release(desc + tile, tot.pack(whole ? WHOLE : TAIL));
         Add before{0, 0, 0};
         if (__shfl_sync(0xffffffffu, runs_in, 0)) {
-            before = oe_look_back(desc, tile, &a.st->error);
-            if (!whole && lane == 0) st128_release(desc + tile, pack(before + tot, WHOLE));
+            before = look_back<Add>(desc, tile, &a.st->error);
+            if (!whole && lane == 0) st128_release(desc + tile, (before + tot).pack(WHOLE));
         }
         if (lane == 0) s_carry = before;
     }
