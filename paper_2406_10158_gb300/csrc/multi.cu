@@ -29,6 +29,7 @@ struct MultiState {
     unsigned long long padded;     // fetch space: chunks rounded up to a power of two
     unsigned int chunk_bits;       // log2 of the number of chunks in it
     unsigned int idle;             // lane groups that found no transaction left
+    unsigned int sort_error;       // GCC_DEVERR_* of the sorts that rank all batches
 };
 
 // Transactions are handed out in chunks of FETCH_CHUNK consecutive ids, the
@@ -132,6 +133,7 @@ __global__ void multi_begin(const ExecArgs* __restrict__ args, DbState* const* _
         }
         ms->fetch = 0;
         ms->idle = 0;
+        ms->sort_error = 0;
         ms->clock.occ_clock = occ;
         ms->clock.to_clock = to;
     }
@@ -151,9 +153,12 @@ __global__ void multi_rq_reset(const ExecArgs* __restrict__ args, uint32_t n) {
     if (i < n && args[i].rq && w < RETRY_QUEUES) args[i].rq[w] = 0;
 }
 
-// Every database continues its own clock from the shared one.
-__global__ void multi_end(DbState* const* __restrict__ own, uint32_t n, const MultiState* ms) {
+// Every database continues its own clock from the shared one.  A sort that
+// failed ranked every batch of the plan, so every batch reports it.
+__global__ void multi_end(const ExecArgs* __restrict__ args, DbState* const* __restrict__ own, uint32_t n,
+                          const MultiState* ms) {
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        if (ms->sort_error) atomicOr(&args[i].st->error, ms->sort_error);
         own[i]->occ_clock = max(own[i]->occ_clock, ms->clock.occ_clock);
         own[i]->to_clock = max(own[i]->to_clock, ms->clock.to_clock);
     }
@@ -410,7 +415,7 @@ gcc_status enqueue(gcc_multi_plan* pl, cudaStream_t st) {
         launches += 1 + radix_sort_launches(8) + 1;
     }
     if (e == cudaSuccess) {
-        multi_end<<<1, 256, 0, st>>>(pl->d_own, pl->n, pl->d_ms);
+        multi_end<<<1, 256, 0, st>>>(pl->d_args, pl->d_own, pl->n, pl->d_ms);
         e = cudaGetLastError();
         launches += 1;
     }
@@ -486,7 +491,7 @@ gcc_status gcc_multi_plan_create(gcc_scheme scheme, const gcc_multi_batch* b, ui
         !alloc((void**)&pl->sort.work, gcc::sort_work_words(items) * 4))
         return bail(fail(GCC_ERR_NOMEM, "cannot allocate the plan"));
     pl->sort.max_items = items;
-    pl->sort.err = &b[0].db->st->error;      // any of the plan's batches: a sort serves them all
+    pl->sort.err = &pl->d_ms->sort_error;    // multi_end tells every batch
 
     std::vector<gcc::ExecArgs> args(n);
     std::vector<gcc::DbState*> own(n);

@@ -1,6 +1,8 @@
 // kernels.cu -- entry points for tests into kernels that the library only
 // launches itself.  One translation unit of the engine is included per PART, so
 // that its internal kernels can be called with buffers of the test's own.
+#include <cstring>
+
 #include <cuda_runtime.h>
 
 #if PART == 0
@@ -66,6 +68,42 @@ int h_multi(gcc_txn_result* r0, gcc_txn_result* r1, unsigned long long* o0, unsi
     gcc::multi_ranks<<<grid_of(total), 256>>>(d, prefix, 2, total, vals);
     const int r = done();
     cudaFree(d);
+    return r;
+}
+// A plan of n databases that begins, has its sort set `sort_error` and ends; errors[i] as database i reports
+// it, which had `own_error` before.  begun: the error word after the beginning.
+int h_plan_error(uint32_t n, unsigned sort_error, unsigned own_error, unsigned* errors, unsigned* begun) {
+    gcc::ExecArgs* args = nullptr;
+    gcc::BatchState* st = nullptr;
+    gcc::DbState* dbs = nullptr;
+    gcc::DbState** own = nullptr;
+    gcc::MultiState* ms = nullptr;
+    cudaMallocManaged(&args, n * sizeof *args);
+    cudaMallocManaged(&st, n * sizeof *st);
+    cudaMallocManaged(&dbs, n * sizeof *dbs);
+    cudaMallocManaged(&own, n * sizeof *own);
+    cudaMallocManaged(&ms, sizeof *ms);
+    if (!args || !st || !dbs || !own || !ms) return -1;
+    std::memset(ms, 0xff, sizeof *ms);
+    std::memset(dbs, 0, n * sizeof *dbs);
+    for (uint32_t i = 0; i < n; ++i) {
+        args[i] = gcc::ExecArgs{};
+        args[i].st = st + i;
+        own[i] = dbs + i;
+    }
+    gcc::multi_begin<<<1, 256>>>(args, own, n, ms, GCC_OCC);
+    int r = done();
+    *begun = ms->sort_error;
+    ms->sort_error = sort_error;
+    for (uint32_t i = 0; i < n; ++i) st[i].error = own_error;
+    gcc::multi_end<<<1, 256>>>(args, own, n, ms);
+    if (!r) r = done();
+    for (uint32_t i = 0; i < n; ++i) errors[i] = st[i].error;
+    cudaFree(args);
+    cudaFree(st);
+    cudaFree(dbs);
+    cudaFree(own);
+    cudaFree(ms);
     return r;
 }
 #elif PART == 3

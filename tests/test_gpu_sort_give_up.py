@@ -169,3 +169,14 @@ def test_order_entry_runs_applied_in_order(lib, n):
         q = q - qty if q >= qty + 10 else q - qty + 91
     assert np.array_equal(host(reads, np.uint64, 2 * n).reshape(n, 2), want)
     assert int(cols[0].cpu().numpy().view(np.uint64)[row]) == q
+
+
+@pytest.mark.parametrize("n", [1, 2, 256])
+def test_every_batch_of_a_plan_reports_its_sort(lib, n):
+    """The sorts that rank a plan's batches rank them all: a wait that gave up is every batch's error."""
+    import ctypes
+    out, begun = (ctypes.c_uint * n)(), ctypes.c_uint(7)
+    assert lib[2].h_plan_error(u32(n), u32(4), u32(1), out, ctypes.byref(begun)) == 0
+    assert begun.value == 0 and list(out) == [5] * n
+    assert lib[2].h_plan_error(u32(n), u32(0), u32(1), out, ctypes.byref(begun)) == 0
+    assert list(out) == [1] * n
