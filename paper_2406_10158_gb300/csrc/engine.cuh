@@ -373,7 +373,8 @@ struct ExecArgs {
     // scheme scratch
     const uint32_t* need;         // DET: per-op wait threshold
     unsigned long long* order_key;// OCC/TO/TicToc: raw commit timestamp per txn
-    uint32_t* seq;                // TicToc: commit sequence number per txn (ties)
+    uint32_t* seq;                // TicToc: commit sequence number per txn (ties); OCC, TO, MVCC:
+                                  // links of the rank lists (order.cu)
     uint32_t det_all;             // DET dataflow: every access waits for all earlier ones
     BatchState* st;
     DbState* dbs;
@@ -586,8 +587,8 @@ cudaError_t det_serial_oe(const ExecArgs& a, const OeTables& T, SortScratch& s, 
 
 // OCC / TO / MVCC: replace raw commit timestamps by dense ranks 0..committed-1.
 struct RankScratch {
-    uint32_t* bits;               // a bit per timestamp, zero between batches
-    uint64_t* counts;             // per word: bits before it << 32 | its bits
+    uint32_t* bits;               // a bit per timestamp, or the heads of lists; zero between batches
+    uint64_t* counts;             // per word: transactions before it << 32 | the word
     uint64_t* desc;               // look-back words of the scan, zero between batches
     uint32_t* ticket;             // its tiles, zero between batches
     uint32_t words;

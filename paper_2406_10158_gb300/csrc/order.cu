@@ -393,19 +393,42 @@ __global__ void det_need(const uint64_t* __restrict__ ops, const uint32_t* __res
 // live in L2 (one bit per attempt), so the three launches cost little more
 // than reading the batch's results: they replace a five-kernel radix sort of
 // (timestamp, transaction), at 2^20 transactions 80 of OCC's 1,480 us.
+// A batch with more timestamps than there are bits (32 per transaction of the
+// largest batch) uses the same words as the heads of lists: word i holds the
+// transactions whose timestamps share the bits from `shift` on, linked through
+// a.seq in no order, the scan counts list lengths, and a rank is the count
+// before the list plus the smaller timestamps in it.  A list is short: the
+// shift is the smallest that fits the words, so it has one transaction on
+// average when the batch is full, and 2^shift at most.  2^20 TO transactions
+// at 50 and at 200 attempts each (kernels of 40 and 156 ms) are ranked in 0.06
+// ms; one block taking a window of the bits at a time took 12 and 38, the sort
+// 0.14.
 // Offsets must fit 32 bits; a batch that used more timestamps than that
 // reports GCC_DEVERR_TS_OVERFLOW.
 __device__ __forceinline__ unsigned long long stamps_used(const ExecArgs& a, int scheme) {
     return scheme == GCC_MVCC ? a.st->ticket
                               : (scheme == GCC_TO ? a.dbs->to_clock : a.dbs->occ_clock) - a.st->ticket_base;
 }
-// Words that hold every timestamp's bit (TO's and MVCC's count from 1).
-__device__ __forceinline__ unsigned long long stamp_words(const ExecArgs& a, int scheme) {
-    return (stamps_used(a, scheme) >> 5) + 1;
+// How the batch is ranked: `words` of the scratch in use, 2^shift timestamps a
+// word, `bits` one bit each or else a list.  (TO's and MVCC's count from 1.)
+struct RankShape {
+    uint32_t words;
+    int shift;
+    bool bits;
+};
+__device__ __forceinline__ RankShape rank_shape(const ExecArgs& a, const RankScratch& r, int scheme) {
+    const unsigned long long n = stamps_used(a, scheme);
+    if ((n >> 5) < r.words) return RankShape{(uint32_t)(n >> 5) + 1, 5, true};
+    int shift = 5;
+    while ((n >> shift) >= r.words) ++shift;
+    return RankShape{(uint32_t)(n >> shift) + 1, shift, false};
+}
+__device__ __forceinline__ unsigned long long stamp(const ExecArgs& a, int scheme, uint32_t t) {
+    return a.order_key[t] - (scheme == GCC_MVCC ? 0ull : a.st->ticket_base);
 }
 __device__ __forceinline__ bool stamp_of(const ExecArgs& a, int scheme, uint32_t t, unsigned long long& d) {
     if (a.results[t].status != GCC_TXN_COMMITTED) return false;
-    d = a.order_key[t] - (scheme == GCC_MVCC ? 0ull : a.st->ticket_base);
+    d = stamp(a, scheme, t);
     return true;
 }
 
@@ -415,10 +438,14 @@ __global__ void rank_mark(const __grid_constant__ ExecArgs a, const RankScratch 
     unsigned long long d;
     if (t >= a.n_txns || !stamp_of(a, scheme, t, d)) return;
     if (d >= 0xffffffffull) atomicOr(&a.st->error, GCC_DEVERR_TS_OVERFLOW);
-    if (stamp_words(a, scheme) <= r.words) atomicOr(&r.bits[d >> 5], 1u << (d & 31));
+    const RankShape s = rank_shape(a, r, scheme);
+    if ((d >> s.shift) >= s.words) return;
+    uint32_t* w = r.bits + (d >> s.shift);
+    if (s.bits) atomicOr(w, 1u << (d & 31));
+    else a.seq[t] = atomicExch(w, t + 1);
 }
 
-// Bits before each word beside the word's bits; leaves `bits` zero.
+// Transactions before each word beside the word; leaves `bits` zero.
 constexpr int RANK_ITEMS = 4;
 __global__ void __launch_bounds__(1024)
 rank_scan(const __grid_constant__ ExecArgs a, const RankScratch r, int scheme) {
@@ -426,20 +453,22 @@ rank_scan(const __grid_constant__ ExecArgs a, const RankScratch r, int scheme) {
     __shared__ uint32_t s_tile;
     __shared__ unsigned long long s_before;
     after_previous();
-    const unsigned long long words = stamp_words(a, scheme);
-    if (words > r.words) return;
+    const RankShape s = rank_shape(a, r, scheme);
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0) s_tile = atomicAdd(r.ticket, 1u);
         __syncthreads();
         const uint32_t tile = s_tile;
         const unsigned long long w0 = (unsigned long long)tile * 1024 * RANK_ITEMS + threadIdx.x * RANK_ITEMS;
-        if ((unsigned long long)tile * 1024 * RANK_ITEMS >= words) return;
-        uint32_t b[RANK_ITEMS], n = 0;
+        if ((unsigned long long)tile * 1024 * RANK_ITEMS >= s.words) return;
+        uint32_t b[RANK_ITEMS], m[RANK_ITEMS], n = 0;
 #pragma unroll
         for (int i = 0; i < RANK_ITEMS; ++i) {
-            b[i] = w0 + i < words ? r.bits[w0 + i] : 0u;
-            n += __popc(b[i]);
+            b[i] = w0 + i < s.words ? r.bits[w0 + i] : 0u;
+            m[i] = 0;
+            if (s.bits) m[i] = __popc(b[i]);
+            else for (uint32_t u = b[i]; u; u = a.seq[u - 1]) ++m[i];
+            n += m[i];
         }
         uint32_t tot;
         uint32_t before = block_exclusive_scan<32>(n, warp_sums, &tot);
@@ -465,62 +494,31 @@ rank_scan(const __grid_constant__ ExecArgs a, const RankScratch r, int scheme) {
         before += (uint32_t)s_before;
 #pragma unroll
         for (int i = 0; i < RANK_ITEMS; ++i)
-            if (w0 + i < words) {
+            if (w0 + i < s.words) {
                 r.counts[w0 + i] = (uint64_t)before << 32 | b[i];
                 if (b[i]) r.bits[w0 + i] = 0u;
-                before += __popc(b[i]);
+                before += m[i];
             }
     }
 }
 
-__device__ __forceinline__ uint32_t rank_of(uint64_t count, uint32_t d) {
-    return (uint32_t)(count >> 32) + __popc((uint32_t)count & ((1u << (d & 31)) - 1u));
-}
-
-// The ranks, and the scan's words left at zero for the next batch.  A batch with
-// more timestamps than `bits` holds (32 per transaction of the largest batch)
-// is ranked by block 0 alone, a window of timestamps at a time: it spent far
-// longer on its attempts than that takes.
+// The ranks, and the scan's words left at zero for the next batch.
 __global__ void __launch_bounds__(256)
 rank_assign(const __grid_constant__ ExecArgs a, const RankScratch r, int scheme) {
-    __shared__ uint32_t warp_sums[32];
     after_previous();
-    const unsigned long long words = stamp_words(a, scheme);
-    if (words <= r.words) {
-        const uint32_t t = blockIdx.x * 256 + threadIdx.x;
-        unsigned long long d;
-        if (t < a.n_txns && stamp_of(a, scheme, t, d)) a.results[t].commit_order = rank_of(r.counts[d >> 5], (uint32_t)d);
-        if (blockIdx.x == 0) {
-            for (uint32_t i = threadIdx.x; i < r.words / (1024 * RANK_ITEMS) + 1; i += 256) r.desc[i] = 0;
-            if (threadIdx.x == 0) *r.ticket = 0;
-        }
-        return;
+    const RankShape s = rank_shape(a, r, scheme);
+    const uint32_t t = blockIdx.x * 256 + threadIdx.x;
+    unsigned long long d;
+    if (t < a.n_txns && stamp_of(a, scheme, t, d) && (d >> s.shift) < s.words) {
+        const uint64_t count = r.counts[d >> s.shift];
+        uint32_t rank = (uint32_t)(count >> 32);
+        if (s.bits) rank += __popc((uint32_t)count & ((1u << (d & 31)) - 1u));
+        else for (uint32_t u = (uint32_t)count; u; u = a.seq[u - 1]) rank += stamp(a, scheme, u - 1) < d;
+        a.results[t].commit_order = rank;
     }
-    if (blockIdx.x != 0) return;
-    const unsigned long long end = words < (1ull << 27) ? words : 1ull << 27;     // 32-bit offsets
-    uint32_t base = 0;
-    for (unsigned long long w0 = 0; w0 < end; w0 += r.words) {
-        const uint32_t m = (uint32_t)(end - w0 < r.words ? end - w0 : r.words);
-        unsigned long long d;
-        for (uint32_t t = threadIdx.x; t < a.n_txns; t += 256)
-            if (stamp_of(a, scheme, t, d) && (d >> 5) >= w0 && (d >> 5) < w0 + m)
-                atomicOr(&r.bits[(d >> 5) - w0], 1u << (d & 31));
-        __threadfence_block();
-        __syncthreads();
-        for (uint32_t i0 = 0; i0 < m; i0 += 256) {
-            const uint32_t i = i0 + threadIdx.x;
-            const uint32_t b = i < m ? atomicExch(&r.bits[i], 0u) : 0u;
-            uint32_t tot;
-            const uint32_t before = block_exclusive_scan<8>(__popc(b), warp_sums, &tot);
-            if (i < m) r.counts[i] = (uint64_t)(base + before) << 32 | b;
-            base += tot;
-        }
-        __threadfence_block();
-        __syncthreads();
-        for (uint32_t t = threadIdx.x; t < a.n_txns; t += 256)
-            if (stamp_of(a, scheme, t, d) && (d >> 5) >= w0 && (d >> 5) < w0 + m)
-                a.results[t].commit_order = rank_of(r.counts[(d >> 5) - w0], (uint32_t)d);
-        __syncthreads();
+    if (blockIdx.x == 0) {
+        for (uint32_t i = threadIdx.x; i < r.words / (1024 * RANK_ITEMS) + 1; i += 256) r.desc[i] = 0;
+        if (threadIdx.x == 0) *r.ticket = 0;
     }
 }
 
