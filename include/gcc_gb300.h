@@ -377,8 +377,11 @@ gcc_status gcc_txn_batch_submit(gcc_db *db, gcc_scheme scheme, const gcc_txn *tx
  * initialisation of the scheme to the completion of every transaction, and
  * the abort rate is aborts per committed transaction (Sec. IV-A, "Metric
  * Selection"); stats carries both, and per-stage times (Sec. III-D,
- * "Measurements and Verification").  The outputs stay owned by the caller.  GCC_ERR_TIMEOUT leaves the batch waitable
- * again.  GCC_ERR_DEVICE when stats.device_error is nonzero (outputs are
+ * "Measurements and Verification").  The outputs stay owned by the caller.
+ * The calling thread polls: for the first 4 ms it only yields its core to
+ * other threads between looks, so each waiter may keep a core busy that long,
+ * after that it sleeps 20 us between them.  GCC_ERR_TIMEOUT leaves the batch
+ * waitable again.  GCC_ERR_DEVICE when stats.device_error is nonzero (outputs are
  * still written). */
 gcc_status gcc_batch_wait(gcc_batch *batch, uint64_t timeout_ns, gcc_txn_result *results,
                           gcc_operand *read_values, gcc_batch_stats *stats,

@@ -781,8 +781,9 @@ gcc_status gcc_batch_wait(gcc_batch* b, uint64_t timeout_ns, gcc_txn_result* res
         if (timeout_ns != UINT64_MAX && waited >= timeout_ns)
             return fail(GCC_ERR_TIMEOUT, "batch still running after %llu ns",
                         (unsigned long long)waited);
-        // a batch of some milliseconds is polled without sleeping: a 20 us sleep
-        // lasts 70 us and more, as much as a small batch's kernel
+        // a batch of some milliseconds is polled without sleeping, as the header
+        // says: a 20 us sleep lasts 70 us and more, as much as a small batch's
+        // kernel
         if (waited > 4000000) std::this_thread::sleep_for(std::chrono::microseconds(20));
         else if (spin > 64) std::this_thread::yield();
     }
