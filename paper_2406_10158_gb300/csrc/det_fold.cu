@@ -347,12 +347,14 @@ fold_tiles(const __grid_constant__ ExecArgs a, const AccessKeys f, const uint32_
     }
 }
 
+// `sort_log2` (CHUNK_LOG2 or more): the ops of one sort.
 template <int FB>
-cudaError_t fold_run(const ExecArgs& a, SortScratch& s, void* scratch, uint32_t& launches, cudaStream_t st) {
+cudaError_t fold_run(const ExecArgs& a, SortScratch& s, void* scratch, uint32_t& launches, cudaStream_t st,
+                     int sort_log2 = SORT_LOG2) {
     const uint64_t n = a.n_ops;
-    const AccessKeys f = access_keys((uint64_t)a.n_fields * a.n_records, n, CHUNK_LOG2, SORT_LOG2, true);
+    const AccessKeys f = access_keys((uint64_t)a.n_fields * a.n_records, n, CHUNK_LOG2, sort_log2, true);
     const DetScratch sc = det_scratch(scratch, n, a.n_txns, CHUNK_LOG2, FT_TILE<16>);
-    const bool one_sort = n <= (1ull << SORT_LOG2);
+    const bool one_sort = n <= (1ull << sort_log2);
     cudaError_t e = launch_det_begin(a, s, sc, f, one_sort, st);
     launches += 1;
     if (e != cudaSuccess || a.n_txns == 0) return e;
@@ -364,8 +366,8 @@ cudaError_t fold_run(const ExecArgs& a, SortScratch& s, void* scratch, uint32_t&
     auto validate = G == 8 ? fold_validate<8> : G == 16 ? fold_validate<16> : fold_validate<32>;
     e = launch_after(validate, grid1, 256, st, a, f, s.k0, s.work, per_block);
     launches += 1;
-    for (uint64_t o0 = 0; o0 < n && e == cudaSuccess; o0 += 1ull << SORT_LOG2) {
-        const uint32_t m = (uint32_t)std::min<uint64_t>(n - o0, 1ull << SORT_LOG2);
+    for (uint64_t o0 = 0; o0 < n && e == cudaSuccess; o0 += 1ull << sort_log2) {
+        const uint32_t m = (uint32_t)std::min<uint64_t>(n - o0, 1ull << sort_log2);
         uint32_t *sk = nullptr, *sv = nullptr;
         e = radix_sort_positions(s, s.k0 + o0, m, f.bits, f.flagged != 0, one_sort, &sk, &sv, st);
         launches += f.passes + (one_sort ? 0 : 1);

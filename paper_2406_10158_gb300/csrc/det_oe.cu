@@ -510,18 +510,13 @@ oe_commit(const __grid_constant__ ExecArgs a, const __grid_constant__ OeTables T
     }
 }
 
-}  // namespace
-
-size_t oe_scratch_bytes(size_t max_ops, size_t max_txns) {
-    return det_scratch(nullptr, max_ops, max_txns, OE_CHUNK_LOG2, OF_TILE).n_zero * 16;
-}
-
-cudaError_t det_serial_oe(const ExecArgs& a, const OeTables& T, SortScratch& s, void* scratch,
-                          uint32_t* list, uint32_t& launches, cudaStream_t st) {
+// `sort_log2` (OE_CHUNK_LOG2 or more): the ops of one sort.
+cudaError_t oe_run(const ExecArgs& a, const OeTables& T, SortScratch& s, void* scratch, uint32_t* list,
+                   uint32_t& launches, cudaStream_t st, int sort_log2 = OE_SORT_LOG2) {
     const uint64_t n = a.n_ops;
-    const AccessKeys f = access_keys(a.n_meta, n, OE_CHUNK_LOG2, OE_SORT_LOG2, true);
+    const AccessKeys f = access_keys(a.n_meta, n, OE_CHUNK_LOG2, sort_log2, true);
     const DetScratch sc = det_scratch(scratch, n, a.n_txns, OE_CHUNK_LOG2, OF_TILE);
-    const bool one_sort = n <= (1ull << OE_SORT_LOG2);
+    const bool one_sort = n <= (1ull << sort_log2);
     cudaError_t e = launch_det_begin(a, s, sc, f, one_sort, st);
     launches += 1;
     if (e != cudaSuccess || a.n_txns == 0) return e;
@@ -529,8 +524,8 @@ cudaError_t det_serial_oe(const ExecArgs& a, const OeTables& T, SortScratch& s, 
     e = launch_after(oe_validate, blocks_for(a.n_txns, (int)per_block), 256, st, a, T, f, s.k0, s.work,
                      per_block);
     launches += 1;
-    for (uint64_t o0 = 0; o0 < n && e == cudaSuccess; o0 += 1ull << OE_SORT_LOG2) {
-        const uint32_t m = (uint32_t)std::min<uint64_t>(n - o0, 1ull << OE_SORT_LOG2);
+    for (uint64_t o0 = 0; o0 < n && e == cudaSuccess; o0 += 1ull << sort_log2) {
+        const uint32_t m = (uint32_t)std::min<uint64_t>(n - o0, 1ull << sort_log2);
         uint32_t *sk = nullptr, *sv = nullptr;
         e = radix_sort_positions(s, s.k0 + o0, m, f.bits, true, one_sort, &sk, &sv, st);
         launches += f.passes + (one_sort ? 0 : 1);
@@ -553,6 +548,17 @@ cudaError_t det_serial_oe(const ExecArgs& a, const OeTables& T, SortScratch& s, 
     e = launch_after(oe_commit, std::min<unsigned>(blocks_for(a.n_txns, 32), 152u * 16u), 256, st, a, T);
     if (e != cudaSuccess) return e;
     return launch_det_finish(a, s, sc, st);
+}
+
+}  // namespace
+
+size_t oe_scratch_bytes(size_t max_ops, size_t max_txns) {
+    return det_scratch(nullptr, max_ops, max_txns, OE_CHUNK_LOG2, OF_TILE).n_zero * 16;
+}
+
+cudaError_t det_serial_oe(const ExecArgs& a, const OeTables& T, SortScratch& s, void* scratch,
+                          uint32_t* list, uint32_t& launches, cudaStream_t st) {
+    return oe_run(a, T, s, scratch, list, launches, st);
 }
 
 }  // namespace gcc

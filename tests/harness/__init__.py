@@ -7,7 +7,7 @@ import subprocess
 from paper_2406_10158_gb300 import build
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-PARTS = 4
+PARTS = 5
 
 
 def load(out_dir):

@@ -13,6 +13,10 @@
 #include "multi.cu"
 #elif PART == 3
 #include "det_oe.cu"
+#include "runtime.cuh"
+#elif PART == 4
+#include "det_fold.cu"
+#include "runtime.cuh"
 #endif
 
 namespace {
@@ -25,6 +29,39 @@ int done() {
 
 extern "C" {
 #if PART == 0
+// A stable sort of (key, position) pairs by the passes with 64-bit descriptors, which otherwise only sorts of 2^30
+// items and more take.  n above 2^19.
+int h_sort_wide(uint32_t* keys, uint32_t n, int bits, int flagged, uint32_t* keys_out, uint32_t* vals_out) {
+    if (gcc::sort_items(n) != gcc::SORT_ITEMS_LARGE) return -1;
+    gcc::SortScratch s{};
+    unsigned* err = nullptr;
+    const size_t words = gcc::SORT_DESC + 2 * gcc::sort_tiles(n) * 256 * 2;
+    cudaMalloc(&s.k1, n * 4ull);
+    cudaMalloc(&s.v0, n * 4ull);
+    cudaMalloc(&s.v1, n * 4ull);
+    cudaMalloc(&s.work, words * 4);
+    cudaMalloc(&err, 4);
+    if (!s.k1 || !s.v0 || !s.v1 || !s.work || !err) return -1;
+    s.k0 = keys;
+    s.err = err;
+    cudaMemset(err, 0, 4);
+    cudaMemset(s.work, 0, words * 4);
+    const gcc::SortPlan plan = gcc::sort_plan(bits);
+    gcc::rs_hist<<<100, gcc::RS_BLOCK>>>(keys, n, bits, plan.passes, plan.digit_bits, s.work + gcc::SORT_HIST);
+    uint32_t *sk = nullptr, *sv = nullptr;
+    cudaError_t e = gcc::rs_passes<uint64_t, gcc::SORT_ITEMS_LARGE>(s, keys, nullptr, n, bits, flagged != 0, &sk, &sv, 0);
+    unsigned bad = 1;
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaMemcpy(&bad, err, 4, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(keys_out, sk, n * 4ull, cudaMemcpyDeviceToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(vals_out, sv, n * 4ull, cudaMemcpyDeviceToDevice);
+    cudaFree(s.k1);
+    cudaFree(s.v0);
+    cudaFree(s.v1);
+    cudaFree(s.work);
+    cudaFree(err);
+    return bad ? -2 : (int)e;
+}
 int h_dense_rank(const uint32_t* sk, const uint32_t* sv, uint32_t n, gcc_txn_result* res) {
     gcc::dense_rank<<<grid_of(n), 256>>>(sk, sv, n, res);
     return done();
@@ -125,6 +162,41 @@ int h_in_order(uint64_t* quantity, uint64_t* ytd, uint64_t* cnt, uint64_t* remot
     const gcc::AccessKeys f = gcc::access_keys(a.n_meta, n, gcc::OE_CHUNK_LOG2, gcc::OE_SORT_LOG2, true);
     gcc::oe_in_order<<<1, 256>>>(a, T, f, sk, sv, 0, 0, n, n_odd, odd);
     return done();
+}
+#endif
+#if PART >= 3
+// The whole pipeline on a database's own scratch, 2^sort_log2 ops to a sort.
+int h_batch_in_parts(gcc_db* db, const gcc_txn* txns, uint32_t n_txns, const uint64_t* ops, const ulonglong2* operands,
+                     uint64_t n_ops, gcc_txn_result* results, ulonglong2* reads, int sort_log2) {
+    gcc::ExecArgs a{};
+    a.txns = txns;
+    a.ops = ops;
+    a.operands = operands;
+    a.n_txns = n_txns;
+    a.n_ops = n_ops;
+    a.results = results;
+    a.reads = reads;
+    a.table = db->table;
+    a.n_records = db->d.n_records;
+    a.n_fields = db->d.n_fields;
+    a.n_meta = db->n_meta;
+    a.n_warehouses = db->d.n_warehouses;
+    a.order_cap = db->d.order_cap;
+    a.max_ops = db->d.max_ops_per_txn;
+    a.st = db->st;
+    a.dbs = db->dbs;
+    uint32_t launches = 0;
+#if PART == 3
+    gcc::OeTables T{};
+    for (int c = 0; c < gcc::rt::OE_NCOLS; ++c) T.c[c] = reinterpret_cast<uint64_t*>(db->cols[c]);
+    T.names = gcc::NameIndex{db->name_idx, db->name_last, db->name_pick};
+    const cudaError_t e = gcc::oe_run(a, T, db->sort, db->fold_seg, db->need, launches, 0, sort_log2);
+#else
+    const cudaError_t e = db->d.field_bytes == 16
+                              ? gcc::fold_run<16>(a, db->sort, db->fold_seg, launches, 0, sort_log2)
+                              : gcc::fold_run<8>(a, db->sort, db->fold_seg, launches, 0, sort_log2);
+#endif
+    return e != cudaSuccess ? (int)e : done();
 }
 #endif
 }
