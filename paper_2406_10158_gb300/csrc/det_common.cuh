@@ -12,8 +12,8 @@ namespace gcc {
 namespace {
 
 // Words of SortScratch::work between the pass tickets and the histograms.
-// The first two are left at zero by the kernel that uses them.
-enum { DW_BEGIN_DONE = 8, DW_UNTILED_ACC, DW_UNTILED, DW_FINISH_TICKET };
+// The first three are left at zero by the kernel that uses them.
+enum { DW_BEGIN_DONE = 8, DW_UNTILED_ACC, DW_FILL_TICKET, DW_UNTILED, DW_FINISH_TICKET };
 
 constexpr uint32_t DET_SPIN_MAX = 1u << 21;
 
@@ -103,9 +103,14 @@ __device__ __forceinline__ bool last_block(uint32_t* counter) {
 // first descriptor area (`zero`, `n_zero` 16-byte words, all of SortScratch::work
 // but the words above) and the pass's own descriptors (`zero2`), and checks that
 // the transactions' op ranges tile ops[0, n_ops) in id order, which the
-// contract asks for.  Where they do not, DW_UNTILED is set and the last block
-// gives every op the key of no record, so that an op outside every range stays
-// out of the access table; the validation pass then overwrites the others'.
+// contract asks for.  Where they do not, DW_UNTILED is set and the blocks that
+// see it give every op the key of no record, a chunk of ops at a time, so that an
+// op outside every range stays out of the access table; the validation pass then
+// overwrites the others'.  (2^24 ops, every seventh transaction left out: 1,399 us
+// for the batch, 2,840 with the last block filling alone; one transaction left
+// out, which one block sees: 2,624 us, 3,169 with chunks of 2^13 ops, whose
+// tickets it waits for one after the other.)
+constexpr uint32_t FILL_CHUNK = 1u << 16;
 __global__ void __launch_bounds__(256)
 det_begin(const __grid_constant__ ExecArgs a, uint32_t* work, ulonglong2* zero, size_t n_zero,
           ulonglong2* zero2, size_t n_zero2, uint32_t* keys, const AccessKeys f) {
@@ -116,7 +121,7 @@ det_begin(const __grid_constant__ ExecArgs a, uint32_t* work, ulonglong2* zero, 
         z.ticket_base = a.dbs->occ_clock;
         *a.st = z;
         for (int w = 0; w < (int)SORT_HIST; ++w)
-            if (w != DW_BEGIN_DONE && w != DW_UNTILED_ACC && w != DW_UNTILED) work[w] = 0;
+            if (w < DW_BEGIN_DONE || w > DW_UNTILED) work[w] = 0;
     }
     const ulonglong2 z2 = make_ulonglong2(0ull, 0ull);
     for (size_t i = i0; i < n_zero; i += stride) zero[i] = z2;
@@ -132,21 +137,31 @@ det_begin(const __grid_constant__ ExecArgs a, uint32_t* work, ulonglong2* zero, 
         if (x.first_op != before) untiled = true;
         if (t + 1 == a.n_txns && (uint64_t)x.first_op + x.n_ops != a.n_ops) untiled = true;
     }
-    if (__syncthreads_or(untiled) && threadIdx.x == 0) atomicOr(work + DW_UNTILED_ACC, 1u);
+    if (__syncthreads_or(untiled)) {
+        __shared__ uint32_t s_chunk;
+        const uint64_t chunks = (a.n_ops + FILL_CHUNK - 1) / FILL_CHUNK;
+        for (;;) {
+            if (threadIdx.x == 0) s_chunk = atomicAdd(work + DW_FILL_TICKET, 1u);
+            __syncthreads();
+            const uint64_t o0 = (uint64_t)s_chunk * FILL_CHUNK;
+            if (s_chunk >= chunks) break;
+            const uint32_t k = f.key(o0, f.none, false);       // one for the whole chunk
+            const uint32_t m = (uint32_t)(a.n_ops - o0 < FILL_CHUNK ? a.n_ops - o0 : FILL_CHUNK);
+            for (uint32_t i = threadIdx.x * 4; i + 4 <= m; i += 1024)
+                *reinterpret_cast<uint4*>(keys + o0 + i) = make_uint4(k, k, k, k);
+            if (threadIdx.x < m % 4) keys[o0 + m / 4 * 4 + threadIdx.x] = k;
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) atomicOr(work + DW_UNTILED_ACC, 1u);
+    }
     if (!last_block(work + DW_BEGIN_DONE)) return;
     const uint32_t bad = *(volatile uint32_t*)(work + DW_UNTILED_ACC);
     __syncthreads();
     if (threadIdx.x == 0) {
         work[DW_UNTILED] = bad;
         work[DW_UNTILED_ACC] = 0;
+        work[DW_FILL_TICKET] = 0;
     }
-    if (!bad) return;
-    for (uint64_t i = threadIdx.x * 4ull; i < a.n_ops; i += 1024)
-        if (i + 4 <= a.n_ops)
-            *reinterpret_cast<uint4*>(keys + i) = make_uint4(f.key(i, f.none, false), f.key(i + 1, f.none, false),
-                                                             f.key(i + 2, f.none, false), f.key(i + 3, f.none, false));
-        else
-            for (uint64_t j = i; j < a.n_ops; ++j) keys[j] = f.key(j, f.none, false);
 }
 
 // Launches det_begin; with one sort for the whole batch (`one_sort`) it also
