@@ -473,7 +473,7 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
     const size_t smem = gu >= 2 ? (size_t)slots * gcc::occ_group_stage_bytes(gu, db->d.max_ops_per_txn)
                                 : (size_t)slots * db->d.max_ops_per_txn * gcc::STAGE_BYTES_PER_OP;
     const int occ = gu >= 2 ? gcc::kv_occ_group_occupancy(db->d.field_bytes, block, smem)
-                    : kv    ? gcc::kv_exec_occupancy(scheme, db->d.field_bytes, block, smem)
+                    : kv    ? gcc::kv_exec_occupancy(scheme, db->d.field_bytes, db->n_meta, block, smem)
                             : gcc::oe_exec_occupancy(scheme, block, smem);
     if (occ <= 0)
         return fail(GCC_ERR_INVALID, "launch shape does not fit an SM (%d threads, %zu B shared)",
@@ -911,7 +911,7 @@ extern "C" gcc_status gcc_autotune(gcc_db* db, gcc_scheme scheme, const gcc_txn*
                 const size_t smem = (size_t)(block / p.lanes_per_txn) * db->d.max_ops_per_txn *
                                     gcc::STAGE_BYTES_PER_OP;
                 const bool kv = db->d.schema == GCC_SCHEMA_KV;
-                const int occ = kv ? gcc::kv_exec_occupancy(scheme, db->d.field_bytes, block, smem)
+                const int occ = kv ? gcc::kv_exec_occupancy(scheme, db->d.field_bytes, db->n_meta, block, smem)
                                    : gcc::oe_exec_occupancy(scheme, block, smem);
                 if (occ <= 0) continue;                          // shape does not fit
                 double rate = 0.0;

@@ -27,7 +27,14 @@ constexpr uint64_t OCC_LOCK = 1ull << 63;
 // read marked to leave L2 first).  OCC keeps 8-byte words: its words are
 // written once per commit, and 4-byte ones measured slower (its kernel took
 // 1,496 against 1,420 us).
+// The words of up to 2^22 records stand 16 bytes apart, a record's whole share of
+// the array: updates of words in one line wait for one another, and the lines
+// still fit L2.  2^18 x 16 ops, 95 % reads, words 4 / 16 bytes apart: 2^20
+// records 536 / 449 us, 2^21 455 / 388, 2^22 398 / 381, 2^23 374 / 430, 2^24
+// 365 / 458.
 constexpr uint32_t TPL_X = 1u << 31;
+constexpr int TPL_SPREAD = 2;         // log2 of the words a spread word takes
+inline bool tpl_spread(uint64_t n_records) { return n_records <= (1u << 22); }
 // TO: one 16-byte word per record, updated with a 128-bit CAS: lo = RTS,
 // hi = WTS (bits 0..62) | dirty (bit 63, the commit bit of Table II).  Table
 // II packs commit bit + 31-bit RTS + 31-bit WTS into 8 bytes, which overflows
@@ -365,7 +372,8 @@ struct ExecArgs {
     uint64_t n_records;
     uint32_t n_fields;
     uint64_t* meta;               // control words: 16 bytes per record, of which 2PL uses
-                                  // the first 4 * n_meta, OCC and DET the first 8 * n_meta
+                                  // the first 4 * n_meta (or one word in four, tpl_spread),
+                                  // OCC and DET the first 8 * n_meta
     uint64_t n_meta;
     int64_t* const* cols;         // order-entry columns (device array of pointers)
     uint32_t n_warehouses;
@@ -463,7 +471,7 @@ constexpr uint32_t STAGE_BYTES_PER_OP = 8 + 8 + 16 + 16 + 8;
 // Key-value execute kernel for one scheme and slot width.
 cudaError_t launch_kv_exec(gcc_scheme scheme, uint32_t field_bytes, const ExecArgs& a,
                            int grid, int block, size_t smem, cudaStream_t s);
-int kv_exec_occupancy(gcc_scheme scheme, uint32_t field_bytes, int block, size_t smem);
+int kv_exec_occupancy(gcc_scheme scheme, uint32_t field_bytes, uint64_t n_records, int block, size_t smem);
 // OCC with group commit on key-value batches (occ_group.cu): unit formation,
 // staging bytes per lane group, launcher and occupancy.
 struct SortScratch;

@@ -87,9 +87,10 @@ struct Lane {
 // SKIPPED: DET only, an invalid transaction's accesses were stepped over
 enum { ABORT = 0, COMMIT = 1, GIVE_UP = 2, SKIPPED = 3 };
 
-// The 32-bit control words of 2PL.
-__device__ __forceinline__ uint32_t* words32(const ExecArgs& a) {
-    return reinterpret_cast<uint32_t*>(a.meta);
+// The 32-bit control word of 2PL.
+template <class Work>
+__device__ __forceinline__ uint32_t* tpl_word(const ExecArgs& a, uint32_t rec) {
+    return reinterpret_cast<uint32_t*>(a.meta) + ((size_t)rec << Work::TPL_SHIFT);
 }
 
 __device__ __forceinline__ bool collapse_loser(const ExecArgs& a, uint32_t rec) {
@@ -253,7 +254,7 @@ __device__ int tpl_attempt(const ExecArgs& a, const Lane& L, const Stage& S, uin
             const uint64_t d = S.desc[j];
             const uint32_t r = Work::rec(a, d);
             if (r != NO_CC) {
-                uint32_t* m = words32(a) + r;
+                uint32_t* m = tpl_word<Work>(a, r);
                 if (!Work::writes(d)) {
                     uint32_t waited = 0;
                     for (uint32_t tries = 0;;) {
@@ -314,7 +315,7 @@ __device__ int tpl_attempt(const ExecArgs& a, const Lane& L, const Stage& S, uin
     for (uint32_t k = 0; k < kmax; ++k)
         if (held >> k & 1) {
             const uint32_t j = L.lig + k * L.G;
-            uint32_t* m = words32(a) + Work::rec(a, S.desc[j]);
+            uint32_t* m = tpl_word<Work>(a, Work::rec(a, S.desc[j]));
             if (!Work::writes(S.desc[j])) { ++L.n_atom; add32_release(m, ~0u); }
             else st_release_u32(m, 0u);
         }

@@ -38,9 +38,11 @@ template <> struct Slot<16> {
     }
 };
 
-template <int FB>
+// TPL: log2 of the distance of 2PL's control words, in words.
+template <int FB, int TPL = 0>
 struct KvWork {
     static constexpr int SCHEMA = GCC_SCHEMA_KV;
+    static constexpr int TPL_SHIFT = TPL;
 
     static __device__ __forceinline__ uint8_t* ptr(const ExecArgs& a, uint64_t d) {
         return a.table + ((uint64_t)op_field(d) * a.n_records + op_key(d)) * FB;

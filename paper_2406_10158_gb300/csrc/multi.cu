@@ -205,38 +205,25 @@ __global__ void multi_ranks(const ExecArgs* __restrict__ args, const uint32_t* _
     if (a.results[t].status == GCC_TXN_COMMITTED) a.results[t].commit_order = p - prefix[i];
 }
 
-template <int SCHEME, int FB>
-int multi_occupancy(int block, size_t smem) {
-    return occupancy_of(multi_kernel<SCHEME, KvWork<FB>>, block, smem);
+// The kernel of a plan, by slot width and for 2PL by the distance of the
+// control words.
+typedef void (*MultiKernel)(const ExecArgs*, const uint32_t*, uint32_t, MultiState*, uint32_t, uint32_t, uint64_t);
+template <int SC, int TPL = 0>
+MultiKernel by_width(uint32_t fb) {
+    return fb == 16 ? multi_kernel<SC, KvWork<16, TPL>> : multi_kernel<SC, KvWork<8, TPL>>;
 }
-
-template <int SCHEME, int FB>
-cudaError_t multi_launch_kernel(const ExecArgs* args, const uint32_t* prefix, uint32_t n,
-                                MultiState* ms, uint32_t lanes, uint32_t max_ops,
-                                uint64_t deadline_ns, int grid, int block, size_t smem,
-                                cudaStream_t st) {
-    // the dynamic shared-memory limit was raised when the plan measured occupancy
-    multi_kernel<SCHEME, KvWork<FB>><<<grid, block, smem, st>>>(args, prefix, n, ms, lanes, max_ops,
-                                                              deadline_ns);
-    return cudaGetLastError();
-}
-
-int occupancy_for(gcc_scheme scheme, uint32_t fb, int block, size_t smem) {
-#define GCC_MULTI_OCC(SC)                                                        \
-    case SC:                                                                     \
-        return fb == 16 ? multi_occupancy<SC, 16>(block, smem)                   \
-                        : multi_occupancy<SC, 8>(block, smem);
+MultiKernel kernel_for(gcc_scheme scheme, uint32_t fb, bool spread) {
     switch (scheme) {
-        GCC_MULTI_OCC(GCC_NO_WAIT_2PL)
-        GCC_MULTI_OCC(GCC_TO)
-        GCC_MULTI_OCC(GCC_OCC)
-        GCC_MULTI_OCC(GCC_TICTOC)
-        GCC_MULTI_OCC(GCC_2PL_WAIT_DIE)
-        GCC_MULTI_OCC(GCC_MVCC)
-        default:
-            return 0;
+        case GCC_NO_WAIT_2PL:
+            return spread ? by_width<GCC_NO_WAIT_2PL, TPL_SPREAD>(fb) : by_width<GCC_NO_WAIT_2PL>(fb);
+        case GCC_2PL_WAIT_DIE:
+            return spread ? by_width<GCC_2PL_WAIT_DIE, TPL_SPREAD>(fb) : by_width<GCC_2PL_WAIT_DIE>(fb);
+        case GCC_TO: return by_width<GCC_TO>(fb);
+        case GCC_OCC: return by_width<GCC_OCC>(fb);
+        case GCC_TICTOC: return by_width<GCC_TICTOC>(fb);
+        case GCC_MVCC: return by_width<GCC_MVCC>(fb);
+        default: return nullptr;
     }
-#undef GCC_MULTI_OCC
 }
 
 // TicToc's serial order over every batch of the plan: three stable passes
@@ -274,6 +261,7 @@ struct gcc_multi_plan {
     int device = 0;
     uint32_t n = 0;
     uint32_t field_bytes = 8;
+    bool spread = false;             // 2PL's control words stand apart
     uint64_t total = 0;
     gcc_exec_params p{};
     std::vector<gcc_db*> dbs;
@@ -356,27 +344,15 @@ gcc_status enqueue(gcc_multi_plan* pl, cudaStream_t st) {
         multi_rq_reset<<<dim3(RETRY_QUEUES / 256, pl->n), 256, 0, st>>>(pl->d_args, pl->n);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
-        const uint32_t lanes = pl->p.lanes_per_txn;
-        const uint64_t dl = std::min<uint64_t>(pl->p.deadline_ns, DEADLINE_MAX_NS);
-        switch (pl->scheme) {
-#define GCC_MULTI_CASE(SC)                                                                         \
-    case SC:                                                                                       \
-        e = pl->field_bytes == 16                                                                  \
-                ? multi_launch_kernel<SC, 16>(pl->d_args, pl->d_prefix, pl->n, pl->d_ms, lanes,     \
-                                              pl->max_ops, dl, pl->grid, pl->block, pl->smem, st)  \
-                : multi_launch_kernel<SC, 8>(pl->d_args, pl->d_prefix, pl->n, pl->d_ms, lanes,      \
-                                             pl->max_ops, dl, pl->grid, pl->block, pl->smem, st);  \
-        break;
-            GCC_MULTI_CASE(GCC_NO_WAIT_2PL)
-            GCC_MULTI_CASE(GCC_TO)
-            GCC_MULTI_CASE(GCC_OCC)
-            GCC_MULTI_CASE(GCC_TICTOC)
-            GCC_MULTI_CASE(GCC_2PL_WAIT_DIE)
-            GCC_MULTI_CASE(GCC_MVCC)
-#undef GCC_MULTI_CASE
-            default:
-                e = cudaErrorInvalidValue;
-                break;
+        const MultiKernel k = kernel_for(pl->scheme, pl->field_bytes, pl->spread);
+        if (k) {
+            // the dynamic shared-memory limit was raised when the plan measured occupancy
+            k<<<pl->grid, pl->block, pl->smem, st>>>(pl->d_args, pl->d_prefix, pl->n, pl->d_ms, pl->p.lanes_per_txn,
+                                                     pl->max_ops,
+                                                     std::min<uint64_t>(pl->p.deadline_ns, DEADLINE_MAX_NS));
+            e = cudaGetLastError();
+        } else {
+            e = cudaErrorInvalidValue;
         }
     }
     uint32_t launches = 3;
@@ -585,7 +561,11 @@ gcc_status gcc_multi_plan_create(gcc_scheme scheme, const gcc_multi_batch* b, ui
     pl->block = (int)p.warps_per_block * 32;
     const uint32_t slots = pl->block / p.lanes_per_txn;
     pl->smem = (size_t)slots * max_ops * gcc::STAGE_BYTES_PER_OP;
-    const int occ = gcc::occupancy_for(scheme, fb, pl->block, pl->smem);
+    uint64_t records = 0;
+    for (uint32_t i = 0; i < n; ++i) records += b[i].db->n_meta;     // they share L2
+    pl->spread = gcc::tpl_spread(records);
+    const gcc::MultiKernel k = gcc::kernel_for(scheme, fb, pl->spread);
+    const int occ = k ? gcc::occupancy_of(k, pl->block, pl->smem) : 0;
     if (occ <= 0) return bail(fail(GCC_ERR_INVALID, "launch shape does not fit an SM"));
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -138,7 +138,7 @@ gcc_status gcc_det_execute_noalloc(void* d_table, uint32_t n_records, uint32_t n
         const int block = 8 * 32;
         const uint32_t slots = block / a.lanes;
         const size_t smem = (size_t)slots * max_ops_per_txn * gcc::STAGE_BYTES_PER_OP;
-        const int occ = gcc::kv_exec_occupancy(GCC_DET, field_bytes, block, smem);
+        const int occ = gcc::kv_exec_occupancy(GCC_DET, field_bytes, n_records, block, smem);
         int sms = 0;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess)

@@ -24,6 +24,7 @@ constexpr uint32_t ITEMS = 100000, CUST = 3000, DIST = 10, LINES = 15;
 
 struct OeWork {
     static constexpr int SCHEMA = GCC_SCHEMA_ORDER_ENTRY;
+    static constexpr int TPL_SHIFT = 0;
 
     static __device__ __forceinline__ uint64_t* col(const ExecArgs& a, int c) {
         return reinterpret_cast<uint64_t*>(a.cols[c]);
