@@ -377,8 +377,8 @@ gcc_status execute_impl(gcc_db* db, gcc_scheme scheme, const gcc_txn* d_txns, ui
     a.need = db->need;
     a.order_key = db->order_key;
     a.seq = db->fold_flags;
-    // MVCC version store: one entry per committed write, in scratch that
-    // the commit ranks only need after the store has been flattened
+    // MVCC version store: one entry per committed write, in the sort's scratch,
+    // which its batches do not use otherwise
     a.mv_wts = db->sort.k0;
     a.mv_next = db->sort.v0;
     a.mv_field = db->sort.k1;

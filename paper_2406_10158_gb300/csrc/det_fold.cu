@@ -208,11 +208,11 @@ __device__ __forceinline__ ulonglong2 slot_plus(ulonglong2 v, Sum s) {
 // by the last of them, after it has acquired the descriptors of the others,
 // which they publish (release) behind that barrier.
 // Bound by the table's random DRAM accesses (a load and, for a changed slot,
-// a write-back each; the part sustains about 39 G of them a second): 2^21 ops
-// over 2.5 GiB take 90 us.  One kernel instead of three (tile totals, tile
-// scan, apply, and a fourth for slots that cross tiles) removes a 16-byte
-// delta per op written and read back; the four took 1.46 ms for 2^24 ops, the
-// eight launches of this one 0.83 ms.
+// a write-back each; a kernel that does nothing else makes 39 G a second of
+// either): 2^21 ops over 2.5 GiB take 84 us.  One kernel instead of three (tile
+// totals, tile scan, apply, and a fourth for slots that cross tiles) removes a
+// 16-byte delta per op written and read back; the four took 1.46 ms for 2^24
+// ops, the eight launches of this one 0.67 ms.
 template <int FB>
 __global__ void __launch_bounds__(FT_THREADS, 4)
 fold_tiles(const __grid_constant__ ExecArgs a, const AccessKeys f, const uint32_t* sk,
