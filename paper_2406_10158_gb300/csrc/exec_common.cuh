@@ -1026,10 +1026,11 @@ __device__ void group_loop(Fetch& F, const Lane& L, const Stage& S, uint32_t M, 
     uint64_t first = 0;
     const ExecArgs* A = nullptr;
     // CUT_WAITS, in one register each: when the warp next looks how many groups
-    // are still at work (low word of the timer), and of the transaction the
-    // number of attempts whose backoff was cut short (bits 0..4, up to 20) and
-    // the latest of them
-    uint32_t look = CUT_WAITS ? (uint32_t)globaltimer() : 0u, cuts = 0;
+    // are still at work (low word of the timer; the same on every lane, which
+    // meet in warp-wide shuffles there), and of the transaction the number of
+    // attempts whose backoff was cut short (bits 0..4, up to 20) and the latest
+    // of them
+    uint32_t look = CUT_WAITS ? __shfl_sync(0xffffffffu, (uint32_t)globaltimer(), 0) : 0u, cuts = 0;
     const uint32_t deadline_64k = (uint32_t)(deadline >> 16);
     const auto past_deadline = [&](uint64_t now_ns) {
         return CUT_WAITS ? (int32_t)((uint32_t)(now_ns >> 16) - deadline_64k) > 0 : now_ns > deadline;
